@@ -951,6 +951,16 @@ static __global__ void __launch_bounds__(32) k_adj_total(double* __restrict__ pa
   if (threadIdx.x == 0) pp[kAdjTotal] = a;
 }
 
+// the same sum, by one warp of the carry sweep (every lane gets it)
+__device__ __forceinline__ float adj_total(const double* __restrict__ partial, int field, const FastArgs& A) {
+  const double* pp = partial + (size_t)field * (kMaxRowBlocks / 2);
+  double a = 0.0;
+  for (int i = threadIdx.x & 31; i < A.zpairs; i += 32) a += pp[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return (float)a;
+}
+
 // ---------------------------------------------------------------------------
 // Recursive column solve, between the row passes: the carry sweep. A block
 // takes 32 columns (one per lane) of one field; its kTriSeg warps cut the G
@@ -971,10 +981,9 @@ static __global__ void __launch_bounds__(32) k_adj_total(double* __restrict__ pa
 // row, X = 0) is U[0][l] = C_l (a y[M-1] + y'[0]): the block's FP64 sum of
 // w_l Re U[0][l] (w = 1 at l = N/2, else 2) is its partial of u[0,0], added in
 // block order by the inverse row pass. Column 0 (b = 2, singular) is the 1D
-// periodic Poisson problem with its mean removed (the reading G[0,0] = 0): the
-// extra warp of block 0 solves it exactly in FP64 and writes it into S.
+// periodic Poisson problem with its mean removed (the reading G[0,0] = 0): one
+// more block per field solves it exactly in FP64 and writes it into S.
 // ---------------------------------------------------------------------------
-constexpr int kTriMaxM = 2112;  // column 0 of the longest supported column
 constexpr int kTriSeg = kTriSegments;  // band segments (warps) per sweep block
 constexpr int kTriTileMaxG = 160;      // bands whose sums a sweep block stages (80 KB)
 
@@ -983,56 +992,71 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_exclusive_scan_d(double v) {
-  const int lane = threadIdx.x & 31;
-  double x = v;
+// Inclusive scan of one FP64 value per thread over NW warps (the whole block when
+// NW > 1, through ws[NW]); the last thread's value, the total, in `total`.
+template <int NW>
+__device__ __forceinline__ double scan_d(double v, double* ws, double& total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const double y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+    const double y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
   }
-  return x - v;
+  if constexpr (NW == 1) {
+    total = __shfl_sync(0xffffffffu, v, 31);
+    return v;
+  }
+  if (lane == 31) ws[warp] = v;
+  __syncthreads();
+  double base = 0.0, t = 0.0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    const double x = ws[w];
+    if (w < warp) base += x;
+    t += x;
+  }
+  __syncthreads();
+  total = t;
+  return v + base;
 }
 
-// Column 0 of one field (warp-wide, FP64): d[r] = u[r+1] - u[r] has
-// d[r] - d[r-1] = f[r] - mean(f); periodicity fixes d[-1] = -sum_r G[r] / M with
-// G the prefix sums; u[0] = 0 (any constant is removed with u[0,0]: column 0
-// adds w_0 U[0][0] = u[0] / N = 0 to it). fcol[p + i] holds column 0 of S row
-// i (bulk copy of pass A's compact copy); each lane walks a contiguous run of
-// torus rows; the solution (1/N folded in) replaces column 0 of S.
-static __device__ __noinline__ void tri_column0(float2* __restrict__ spec, float* fcol, int field,
-                                                const FastArgs& A, float x0) {
-  const int lane = threadIdx.x & 31;
-  float2* col = spec + (size_t)field * A.srows * A.ldY;
-  const int nr = min(A.srows, A.M - A.p);  // S rows on the torus
-  for (int r = lane; r < A.M; r += 32)
-    if (r < A.p || r >= A.p + nr) fcol[r] = 0.0f;
-  if (lane == 0) fcol[0] = x0;  // torus row 0 (the adjoint's -(sum grad_out) e_00; else 0)
-  __syncwarp();
-  const int run = (A.M + 31) / 32;
-  const int r0 = min(lane * run, A.M), r1 = min(r0 + run, A.M);
-  double s0 = 0.0;
-  for (int r = r0; r < r1; ++r) s0 += (double)fcol[r];
-  const double mean = warp_sum_d(s0) * A.invM;
-  const double off = warp_exclusive_scan_d(s0 - mean * (double)(r1 - r0));
-  double Gr = off, Gs = 0.0;
+// Column 0 of one field (FP64, by NW warps): d[r] = u[r+1] - u[r] has
+// d[r] - d[r-1] = f[r] - mean(f); periodicity fixes d[-1] = D = -sum_r G[r] / M
+// with G the prefix sums of f - mean(f); u[0] = 0 (any constant is removed with
+// u[0,0]: column 0 adds w_0 U[0][0] = u[0] / N = 0 to it). f(r) gives torus row
+// r's value; each thread takes a contiguous run of rows: one pass for its sums
+// P = sum f and Q = sum of f's running sums, two scans over the threads, one pass
+// that rebuilds u. put(r, u[r] / N) for every torus row. FP64 runs at a small
+// fraction of the FP32 rate here, so the passes do eight FP64 instructions a
+// row; one warp at thirteen a row, on the sweep's critical path, was 12 of the
+// 24 us of a sweep of 3 fields of 801x1200 and 36 of 101 for 2048 of 256x256.
+template <int NW, class F, class Put>
+__device__ __forceinline__ void column0_solve(F f, Put put, double* ws, int M, double invM, double invN) {
+  const int run = (M + 32 * NW - 1) / (32 * NW);
+  const int me = NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int r0 = min(me * run, M), r1 = min(r0 + run, M), n = r1 - r0;
+  double P = 0.0, Q = 0.0;  // sum of f, sum over the run's rows of the running sum
   for (int r = r0; r < r1; ++r) {
-    Gr += (double)fcol[r] - mean;
-    Gs += Gr;
+    P += (double)f(r);
+    Q += P;
   }
-  const double D = -warp_sum_d(Gs) * A.invM;
-  double u = warp_exclusive_scan_d(D * (double)(r1 - r0) + Gs);
-  const double invN = A.invN;
-  Gr = off;
+  double sum, gsum;
+  const double Pi = scan_d<NW>(P, ws, sum);
+  const double mean = sum * invM;
+  const double off = (Pi - P) - mean * (double)r0;                       // G just above the run
+  const double Gs = Q + (double)n * (off - mean * (0.5 * (double)(n + 1)));  // sum of G over the run
+  const double Gi = scan_d<NW>(Gs, ws, gsum);
+  const double D = -gsum * invM;
+  double u = ((Gi - Gs) + D * (double)r0) * invN, g = (off + D) * invN;
+  const double mN = mean * invN;
   for (int r = r0; r < r1; ++r) {
-    const int i = r - A.p;
-    if (i >= 0 && i < nr) col[(size_t)i * A.ldY] = make_float2((float)(u * invN), 0.0f);
-    Gr += (double)fcol[r] - mean;
-    u += D + Gr;
+    put(r, (float)u);
+    g += fma((double)f(r), invN, -mN);
+    u += g;
   }
 }
 
-static __global__ void __launch_bounds__(32 * (kTriSeg + 1)) k_tri_carries(float2* __restrict__ spec,
+static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __restrict__ spec,
                                                                           float2* __restrict__ tri,
                                                                           const float* __restrict__ cc,
                                                                           const float* __restrict__ powc,
@@ -1040,40 +1064,56 @@ static __global__ void __launch_bounds__(32 * (kTriSeg + 1)) k_tri_carries(float
   __shared__ float2 seg_e[kTriSeg][kTriCols], seg_q[kTriSeg][kTriCols];  // segment totals, then carries
   __shared__ float2 y0s[kTriCols];
   __shared__ float yls[2 * kTriCols];
-  __shared__ __align__(16) float fcol[kTriMaxM + 4];  // block 0: column 0 of S (compact copy)
-  __shared__ __align__(8) uint64_t bar, tbar;
+  __shared__ __align__(8) uint64_t tbar;
+  __shared__ float sadj_s;
+  __shared__ double ws[kTriSeg];
   extern __shared__ __align__(16) float2 tile[];  // the block's band sums when they fit (staged)
+  const int nkb = gridDim.x - 1;  // column blocks; one more block for column 0
   const int kb = blockIdx.x, field = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = kb * kTriCols + lane;
   const bool col_ok = k >= 1 && k < A.Nh;
-  // the adjoint's z has -(sum grad_out) at torus (0, 0): -s in every column of row 0
-  const float sadj = A.adj ? (float)partial[(size_t)field * (kMaxRowBlocks / 2) + kAdjTotal] : 0.0f;
+  if (kb == nkb) {
+    const float sadj = A.adj ? adj_total(partial, field, A) : 0.0f;  // (every warp for itself)
+    const int nr = min(A.srows, A.M - A.p);
+    const float* c0 = tri_col0(tri, field, A);
+    float2* col = spec + (size_t)field * A.srows * A.ldY;
+    column0_solve<kTriSeg>(
+        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldg(c0 + (r - A.p)) : 0.0f); },
+        [&](int r, float u) {
+          if (r >= A.p && r < A.p + nr) col[(size_t)(r - A.p) * A.ldY] = make_float2(u, 0.0f);
+        },
+        ws, A.M, A.invM, A.invN);
+    return;
+  }
   const float2* gsums = tri_sums(tri, field, A) + (size_t)kb * 2 * A.G * kTriCols;  // [g][2][32], contiguous
   const bool staged = A.G <= kTriTileMaxG;
   const float2* sums = (staged ? tile : gsums) + lane;
   float2* carry = tri + (size_t)field * A.tri_field + k;  // [g][2][ldY]
-  // column 0's compact copy for block 0's extra warp, in flight during the sweeps
-  const int nr = min(A.srows, A.M - A.p);
-  const unsigned cbytes = (unsigned)((nr * sizeof(float) + 15) & ~(size_t)15);
-  if (kb == 0 && tid == 32 * kTriSeg) {
-    mbar_init(&bar, 1);
-    mbar_expect_tx(&bar, cbytes);
-    bulk_copy(fcol + A.p, tri_col0(tri, field, A), cbytes, &bar);
-  }
   if (staged) {  // the whole tile of band sums by one bulk copy
     if (tid == 0) {
       mbar_init(&tbar, 1);
       bulk_load(tile, gsums, (unsigned)(2 * A.G * kTriCols * sizeof(float2)), &tbar);
+    }
+    if (A.adj && warp == 1) {
+      const float t = adj_total(partial, field, A);
+      if (lane == 0) sadj_s = t;
     }
     __syncthreads();
     const bool landed = mbar_wait(&tbar, 0);
     if (__syncthreads_or(!landed)) {  // the copy never completed: report, let it drain, stop
       if (tid == 0) atomicExch(A.err, kErrBulkWait);
       mbar_wait(&tbar, 0);
-      if (kb == 0 && tid == 32 * kTriSeg) mbar_wait(&bar, 0);
       return;
     }
+  } else if (A.adj) {
+    if (warp == 1) {
+      const float t = adj_total(partial, field, A);
+      if (lane == 0) sadj_s = t;
+    }
+    __syncthreads();
   }
+  // the adjoint's z has -(sum grad_out) at torus (0, 0): -s in every column of row 0
+  const float sadj = A.adj ? sadj_s : 0.0f;
   float4 c03 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), c47 = c03;
   if (col_ok) {
     c03 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8));
@@ -1186,25 +1226,16 @@ static __global__ void __launch_bounds__(32 * (kTriSeg + 1)) k_tri_carries(float
       done = atomicAdd(reinterpret_cast<unsigned*>(pp + kTriCnt), 1u);
     }
     done = __shfl_sync(0xffffffffu, done, 0);
-    if (done == (unsigned)gridDim.x - 1) {
+    if (done == (unsigned)nkb - 1) {
       // the field's last sweep block: u[0,0] from every block's partial,
       // lane-strided then a fixed shuffle tree (the same order on every call)
       __threadfence();
       double s2 = 0.0;
-      for (int i = lane; i < (int)gridDim.x; i += 32) s2 += __ldcg(pp + i);
+      for (int i = lane; i < nkb; i += 32) s2 += __ldcg(pp + i);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s2 += __shfl_down_sync(0xffffffffu, s2, o);
       if (lane == 0) pp[kTriU00] = s2;
     }
-  }
-  if (warp == kTriSeg && kb == 0) {
-    const bool landed = mbar_wait(&bar, 0);
-    if (!landed) {  // the copy never completed: report, let it drain, stop
-      if (lane == 0) atomicExch(A.err, kErrBulkWait);
-      mbar_wait(&bar, 0);
-      return;
-    }
-    tri_column0(spec, fcol, field, A, -sadj);
   }
 }
 
@@ -1212,9 +1243,8 @@ static __global__ void __launch_bounds__(32 * (kTriSeg + 1)) k_tri_carries(float
 // block of 32 columns), one column per lane, all of the block's band sums in
 // registers (one round of loads per direction), each direction swept from a
 // zero carry and then from the true carries, as above; no shared-memory
-// staging and no block barriers. The warp of column block 0 then solves
-// column 0 exactly (fcol: M + 4 floats of shared memory per warp), and each
-// field's last warp to finish combines the u[0,0] partials.
+// staging and no block barriers. One more warp per field solves column 0 exactly,
+// and each field's last warp to finish combines the u[0,0] partials.
 constexpr int kTriRegG = 32;
 constexpr int kTriRegWarps = 8;
 static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg(float2* __restrict__ spec,
@@ -1222,16 +1252,27 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
                                                                            const float* __restrict__ cc,
                                                                            double* __restrict__ partial, FastArgs A,
                                                                            int nkb) {
-  extern __shared__ __align__(16) float fcols[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int task = blockIdx.x * kTriRegWarps + warp;
-  if (task >= A.nf * nkb) return;
-  const int field = task / nkb, kb = task - field * nkb;
+  if (task >= A.nf * (nkb + 1)) return;
+  const int field = task / (nkb + 1), kb = task - field * (nkb + 1);
   const int k = kb * kTriCols + lane;
   const bool col_ok = k >= 1 && k < A.Nh;
   const int G = A.G;
   // the adjoint's z has -(sum grad_out) at torus (0, 0): -s in every column of row 0
-  const float sadj = A.adj ? (float)partial[(size_t)field * (kMaxRowBlocks / 2) + kAdjTotal] : 0.0f;
+  const float sadj = A.adj ? adj_total(partial, field, A) : 0.0f;
+  if (kb == nkb) {
+    const int nr = min(A.srows, A.M - A.p);
+    const float* c0 = tri_col0(tri, field, A);
+    float2* col = spec + (size_t)field * A.srows * A.ldY;
+    column0_solve<1>(
+        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldg(c0 + (r - A.p)) : 0.0f); },
+        [&](int r, float u) {
+          if (r >= A.p && r < A.p + nr) col[(size_t)(r - A.p) * A.ldY] = make_float2(u, 0.0f);
+        },
+        nullptr, A.M, A.invM, A.invN);
+    return;
+  }
   const float2* sums = tri_sums(tri, field, A) + (size_t)kb * 2 * G * kTriCols + lane;  // [g][2][32]
   float2* carry = tri + (size_t)field * A.tri_field + k;                                 // [g][2][ldY]
   double acc = 0.0;
@@ -1290,14 +1331,6 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
   }
   acc = warp_sum_d(acc);
   double* pp = partial + (size_t)field * (kMaxRowBlocks / 2);
-  if (kb == 0) {  // column 0, from the compact copy of S's column 0
-    float* fcol = fcols + (size_t)warp * (A.M + 4);
-    const int nr = min(A.srows, A.M - A.p);
-    const float* c0 = tri_col0(tri, field, A);
-    for (int i = lane; i < nr; i += 32) fcol[A.p + i] = c0[i];
-    __syncwarp();
-    tri_column0(spec, fcol, field, A, -sadj);
-  }
   if (A.adj) return;  // u[0,0]: the adjoint has no offset
   unsigned done = 0;
   if (lane == 0) {
@@ -2125,7 +2158,7 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   A.tri_field = P->tri_field;
   const int nkb = (P->Nh + kTriCols - 1) / kTriCols;
   if ((size_t)2 * RS::F * A.ldY > (size_t)RS::F * RS::NP || A.zpairs > kAdjTotal ||
-      (size_t)A.srows * A.ldY > P->spec_field || nkb > kTriCnt || P->M > kTriMaxM)
+      (size_t)A.srows * A.ldY > P->spec_field || nkb > kTriCnt)
     return cudaErrorInvalidConfiguration;
   static std::mutex mu;
   static int slots_a = 0, slots_c = 0;
@@ -2141,7 +2174,7 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
       if ((e = fast_setup(k_fast_rows_adj<RS, T, true>, RS::THREADS, RS::smem_bytes_adj_tri(), &slots_c)) !=
           cudaSuccess)
         return e;
-      if ((e = fast_setup(k_tri_carries, 32 * (kTriSeg + 1), (size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2),
+      if ((e = fast_setup(k_tri_carries, 32 * kTriSeg, (size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2),
                           &unused)) != cudaSuccess)
         return e;
       ready = true;
@@ -2157,16 +2190,13 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
   double* pd = reinterpret_cast<double*>(bf.partial);
-  k_adj_total<<<nf, 32, 0, st>>>(pd, A.zpairs);
-  P->prof.launches[1] += 1;  // a second launch in this pass
-  if (A.G <= kTriRegG && (size_t)kTriRegWarps * (P->M + 4) * sizeof(float) <= 48 * 1024) {
-    const int tasks = nf * nkb;
-    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps,
-                        (size_t)kTriRegWarps * (P->M + 4) * sizeof(float), st>>>(bf.spec, bf.tri, P->colcoef_h, pd, A,
-                                                                                nkb);
+  if (A.G <= kTriRegG) {
+    const int tasks = nf * (nkb + 1);
+    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps, 0, st>>>(
+        bf.spec, bf.tri, P->colcoef_h, pd, A, nkb);
   } else {
     const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb, nf), 32 * (kTriSeg + 1), tsm, st>>>(bf.spec, bf.tri, P->colcoef_h, P->powc_h, pd, A);
+    k_tri_carries<<<dim3(nkb + 1, nf), 32 * kTriSeg, tsm, st>>>(bf.spec, bf.tri, P->colcoef_h, P->powc_h, pd, A);
   }
   prof_end(P, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -2257,7 +2287,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
       }
       if constexpr (MODE != 2) {
         int unused_k = 0;
-        if ((e = fast_setup(k_tri_carries, 32 * (kTriSeg + 1), (size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2),
+        if ((e = fast_setup(k_tri_carries, 32 * kTriSeg, (size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2),
                             &unused_k)) != cudaSuccess)
           return e;
         if ((e = fast_setup(k_fast_rows_inv<RS, T, true, false>, RS::THREADS, RS::smem_bytes_tri_inv(), &slots_tc)) !=
@@ -2343,14 +2373,13 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
   const int nkb = (P->Nh + kTriCols - 1) / kTriCols;  // column blocks of the sweep (u[0,0] partials)
-  if (tri && A.G <= kTriRegG && (size_t)kTriRegWarps * (P->M + 4) * sizeof(float) <= 48 * 1024) {
-    const int tasks = nf * nkb;
-    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps,
-                        (size_t)kTriRegWarps * (P->M + 4) * sizeof(float), st>>>(
+  if (tri && A.G <= kTriRegG) {
+    const int tasks = nf * (nkb + 1);
+    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps, 0, st>>>(
         bf.spec, bf.tri, P->colcoef, reinterpret_cast<double*>(bf.partial), A, nkb);
   } else if (tri) {
     const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb, nf), 32 * (kTriSeg + 1), tsm, st>>>(bf.spec, bf.tri, P->colcoef, P->powc,
+    k_tri_carries<<<dim3(nkb + 1, nf), 32 * kTriSeg, tsm, st>>>(bf.spec, bf.tri, P->colcoef, P->powc,
                                                                    reinterpret_cast<double*>(bf.partial), A);
   } else if constexpr (kCols) {
     if (MODE == 2) {

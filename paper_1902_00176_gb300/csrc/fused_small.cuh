@@ -306,9 +306,11 @@ __global__ void __launch_bounds__(S::THREADS, 2) k_fused_small(const T* __restri
       }
     }
     __syncwarp();
-    FastArgs A1 = A;
-    A1.ldY = 1;  // the solution goes to col0[i], i < nr
-    tri_column0(col0, fcol, 0, A1, 0.0f);
+    column0_solve<1>([&](int r) { return r >= A.p && r < A.p + nr ? fcol[r] : 0.0f; },
+                     [&](int r, float u) {
+                       if (r >= A.p && r < A.p + nr) col0[r - A.p] = make_float2(u, 0.0f);
+                     },
+                     nullptr, A.M, A.invM, A.invN);
   }
   __syncthreads();  // tile_u complete
   if (tid < 32) {
