@@ -660,26 +660,77 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd(const
 }
 
 // ---------------------------------------------------------------------------
-// pass L folded into pass A (gradient input): the 2F gx rows and 2F + 1 gy rows
-// an item needs (gy from the row above its first pair) arrive as two bulk
-// copies into the exchange buffers, and each thread forms its packed values
-// L[2 pair][j] + i L[2 pair + 1][j] (Eq. 3) from shared memory with the same
-// arithmetic as pass L, so the packed rows never go through HBM. The rest is
-// k_fast_rows_fwd. The next item's rows are requested once this item's
-// spectrum is stored (the staging area spans both exchange buffers).
-// ADJ: the adjoint's first step instead, z = Crop^T(grad_out) from the 2F
-// staged rows of grad_out, with each row pair's FP64 sum written where pass B
-// reads it for the -(sum grad_out) e_00 term (as k_fast_div<T, 2>).
-// Requires W sizeof(T) to be a multiple of 16 and the staging to fit
-// (fused_div_fits).
+// pass L folded into pass A: the input rows an item needs arrive by bulk copy in
+// the exchange buffers and each thread forms its packed values
+// L[2 pair][j] + i L[2 pair + 1][j] from shared memory with the same arithmetic
+// as pass L, so the packed rows never go through HBM. IN = kInGrad: 2F gx rows
+// and 2F + 1 gy rows (gy from the row above the item's first pair), Eq. 3;
+// kInLap: 2F rows of a given Laplacian; kInAdj: the adjoint's first step,
+// z = Crop^T(grad_out) from 2F rows of grad_out, with each row pair's FP64 sum
+// written where pass B reads it for the -(sum grad_out) e_00 term (as
+// k_fast_div<T, 2>). The rest is k_fast_rows_fwd. The next item's rows are
+// requested once this item's spectrum is stored (the staging area spans both
+// exchange buffers).
+// The rows of an item are one contiguous run of global memory, so rows of any
+// length are staged: the copy starts at the 16-byte boundary at or below the
+// first element and ends at the one at or above the last, and the row pointers
+// start at the remainder. Only a run that ends at the end of the whole input
+// stops at the boundary below, and its last elements (fewer than 16 bytes) are
+// loaded one by one.
 // ---------------------------------------------------------------------------
+enum FwdIn { kInGrad = 0, kInLap = 1, kInAdj = 2 };
+
+// shared memory of one staged run of n elements: at most 15 bytes of another
+// run in front, whole 16-byte units
+template <typename T>
+__host__ __device__ constexpr size_t run_bytes(size_t n) {
+  return (n * sizeof(T) + 15 + 15) / 16 * 16;
+}
+// the item's input rows as staged: gradient 2F gx rows, then 2F + 1 gy rows;
+// Laplacian and adjoint 2F rows
 template <class S, typename T>
-__host__ __device__ constexpr size_t fused_stage_bytes(int W) {
-  return (size_t)(4 * S::F + 1) * W * sizeof(T);
+__host__ __device__ constexpr size_t fused_stage_bytes(int W, int in = kInGrad) {
+  return run_bytes<T>((size_t)2 * S::F * W) + (in == kInGrad ? run_bytes<T>((size_t)(2 * S::F + 1) * W) : 0);
 }
 template <class S>
 __host__ __device__ constexpr size_t fused_exchange_bytes() {
   return (size_t)(S::F * S::NP + S::F * S::NO) * sizeof(float2);
+}
+
+// a run of n > 0 elements at src of an input that ends at `end`, as it is copied
+template <typename T>
+struct Run {
+  const char* from;  // 16-byte aligned, at or below src
+  unsigned bytes;    // whole 16-byte units copied
+  int lead;          // elements between `from` and src
+  int tail;          // last elements of the run that the copy does not reach
+  __device__ __forceinline__ Run(const T* src, unsigned n, const T* end) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src), e = a + (uintptr_t)n * sizeof(T), b = a & ~(uintptr_t)15;
+    uintptr_t stop = (e + 15) & ~(uintptr_t)15;
+    if (stop > reinterpret_cast<uintptr_t>(end)) stop = e & ~(uintptr_t)15;
+    from = reinterpret_cast<const char*>(b);
+    bytes = stop > b ? (unsigned)(stop - b) : 0u;
+    lead = (int)((a - b) / sizeof(T));
+    tail = e > stop ? (int)((e - (stop > a ? stop : a)) / sizeof(T)) : 0;
+  }
+};
+
+// Store n contiguous elements from shared memory to dst, by one warp: the
+// 16-byte units of dst that the run covers by bulk copy, the elements before
+// and after them one by one. src is at dst's remainder from a 16-byte boundary.
+// The caller's lane 0 waits for the copy; the lanes' reads of shared memory are
+// ordered before later asynchronous writes to it.
+template <typename T>
+__device__ __forceinline__ void store_run(T* dst, const T* src, unsigned n, int lane) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(dst), e = a + (uintptr_t)n * sizeof(T);
+  uintptr_t b = (a + 15) & ~(uintptr_t)15, stop = e & ~(uintptr_t)15;
+  if (stop < b) b = stop = e;  // no whole unit
+  const unsigned head = (unsigned)((b - a) / sizeof(T)), last = (unsigned)((stop - a) / sizeof(T));
+  if (lane == 0 && stop > b) bulk_store(dst + head, src + head, (unsigned)(stop - b));
+  if (lane < (int)head) dst[lane] = src[lane];
+  if (lane < (int)(n - last)) dst[last + lane] = src[last + lane];
+  fence_proxy_async_smem();
+  __syncwarp();
 }
 
 // EDIT = kEditThreshold (Sec. 3.2.3) zeroes, in the staged rows, every pixel whose
@@ -687,7 +738,7 @@ __host__ __device__ constexpr size_t fused_exchange_bytes() {
 // the chunk's fields), with the keep/drop decision of the standalone threshold
 // kernel, before the divergence is formed; the gy row above the item takes its
 // decision from gx of that row, read from global memory ahead of the staging.
-template <class S, typename T, bool ADJ, bool TRI, int EDIT = kEditNone>
+template <class S, typename T, int IN, bool TRI, int EDIT = kEditNone>
 __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(const T* __restrict__ gx,
                                                                      const T* __restrict__ gy,
                                                                      float2* __restrict__ spec,
@@ -696,14 +747,17 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
                                                                      float2* __restrict__ tri,
                                                                      const float* __restrict__ cc,
                                                                      const float* __restrict__ t2s = nullptr) {
-  static_assert(EDIT == kEditNone || (EDIT == kEditThreshold && !ADJ), "only the threshold edit is staged");
+  constexpr bool ADJ = IN == kInAdj;
+  static_assert(EDIT == kEditNone || (EDIT == kEditThreshold && IN == kInGrad), "only the threshold edit is staged");
   extern __shared__ __align__(16) float2 sm[];
   float2* tw2 = sm;
   float2* buf = sm + S::R1 * S::R2;
   float2* buf2 = buf + S::F * S::NP;
   constexpr int RW = 2 * S::F;  // image rows per item
-  T* sgx = reinterpret_cast<T*>(buf);  // gx rows (ADJ: grad_out rows) r0 .. r0 + RW - 1
-  T* sgy = sgx + (size_t)RW * A.W;     // gy rows r0 - 1 .. r0 + RW - 1
+  static_assert((S::R1 * S::R2) % 2 == 0, "the staging area is 16-byte aligned");
+  // gx rows (else the only input's rows) r0 .. r0 + RW - 1; gy rows from the one above
+  T* const stx = reinterpret_cast<T*>(buf);
+  T* const sty = reinterpret_cast<T*>(reinterpret_cast<char*>(buf) + run_bytes<T>((size_t)RW * A.W));
   __shared__ __align__(8) uint64_t bar;
   __shared__ float2 red[ADJ ? S::F * S::T : 1];  // ADJ: per-thread compensated sums (sum, error) of the row pairs
   const int tid = threadIdx.x;
@@ -719,34 +773,48 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
   const bool uact = tid < S::F * S::T;
   const int items = A.nf * A.ngroups;
   const size_t fe = (size_t)A.H * A.W;
-  // one thread: stage the gradient rows of item w (prefetch: only start
-  // fetching the same rows into L2, for the copy one item later)
+  const T* const xend = gx + (size_t)A.nf * fe;
+  // rows of whole 16-byte units start every run at a boundary (so do the fields)
+  const bool whole = (A.W * sizeof(T)) % 16 == 0;
+  const T* const yend = IN == kInGrad ? gy + (size_t)A.nf * fe : nullptr;
+  // the runs of item w: rows r0 .. r0 + nx - 1 of gx (nx may be 0), rows y0 .. y1 - 1 of gy
+  auto rows_x = [&](int r0) { return (A.H - r0) < RW ? (A.H - r0) : RW; };
+  auto run_x = [&](int field, int r0, int nx) { return Run<T>(gx + field * fe + (size_t)r0 * A.W, (unsigned)(nx * A.W), xend); };
+  auto run_y = [&](int field, int r0) {
+    const int y0 = r0 > 0 ? r0 - 1 : 0, y1 = (A.H < r0 + RW) ? A.H : r0 + RW;
+    return Run<T>(gy + field * fe + (size_t)y0 * A.W, (unsigned)((y1 - y0) * A.W), yend);
+  };
+  // one thread: stage the input rows of item w (prefetch: only start fetching
+  // the same rows into L2, for the copy one item later)
   auto issue = [&](int w, bool prefetch) {
     const int field = w / A.ngroups, g = w - field * A.ngroups;
-    const int r0 = g * RW;
-    const int nx = (A.H - r0) < RW ? (A.H - r0) : RW;             // gx rows r0 .. r0 + nx - 1 (nx may be 0)
-    const int y0 = r0 > 0 ? r0 - 1 : 0, y1 = (A.H < r0 + RW) ? A.H : r0 + RW;  // gy rows y0 .. y1 - 1
-    const unsigned row = (unsigned)(A.W * sizeof(T));
-    const T* xs = gx + field * fe + (size_t)r0 * A.W;
-    const T* ys = gy + field * fe + (size_t)y0 * A.W;
+    const int r0 = g * RW, nx = rows_x(r0);  // (with the recursive column solve the last band may hold no row)
+    const char* xs = nullptr;
+    const char* ys = nullptr;
+    unsigned xb = 0, yb = 0;
+    if (nx > 0) {
+      const Run<T> q = run_x(field, r0, nx);
+      xs = q.from;
+      xb = q.bytes;
+    }
+    if constexpr (IN == kInGrad) {
+      const Run<T> q = run_y(field, r0);
+      ys = q.from;
+      yb = q.bytes;
+    }
     if (prefetch) {
-      if (nx > 0) l2_prefetch(xs, (unsigned)nx * row);
-      if (!ADJ) l2_prefetch(ys, (unsigned)(y1 - y0) * row);
+      if (xb) l2_prefetch(xs, xb);
+      if (yb) l2_prefetch(ys, yb);
       return;
     }
-    if constexpr (ADJ) {  // (with the recursive column solve the last band may hold no row of grad_out)
-      mbar_expect_tx(&bar, (unsigned)(nx > 0 ? nx : 0) * row);
-      if (nx > 0) bulk_copy(sgx, xs, (unsigned)nx * row, &bar);
+    mbar_expect_tx(&bar, xb + yb);
+    if (IN != kInAdj && A.l2res) {  // read once: first out of the L2, so that the spectrum stays
+      const uint64_t pol = l2_policy_evict_first();
+      if (xb) bulk_copy_hint(stx, xs, xb, &bar, pol);
+      if (yb) bulk_copy_hint(sty, ys, yb, &bar, pol);
     } else {
-      mbar_expect_tx(&bar, (unsigned)(nx > 0 ? nx : 0) * row + (unsigned)(y1 - y0) * row);
-      if (A.l2res) {  // read once: first out of the L2, so that the spectrum stays
-        const uint64_t pol = l2_policy_evict_first();
-        if (nx > 0) bulk_copy_hint(sgx, xs, (unsigned)nx * row, &bar, pol);
-        bulk_copy_hint(sgy + (size_t)(y0 - (r0 - 1)) * A.W, ys, (unsigned)(y1 - y0) * row, &bar, pol);
-      } else {
-        if (nx > 0) bulk_copy(sgx, xs, (unsigned)nx * row, &bar);
-        bulk_copy(sgy + (size_t)(y0 - (r0 - 1)) * A.W, ys, (unsigned)(y1 - y0) * row, &bar);
-      }
+      if (xb) bulk_copy(stx, xs, xb, &bar);
+      if (yb) bulk_copy(sty, ys, yb, &bar);
     }
   };
   if (tid == 0) mbar_init(&bar, 1);
@@ -776,6 +844,27 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
       mbar_wait(&bar, phase);
       return;
     }
+    // the staged rows: sgx row i is image row r0 + i, sgy row i image row r0 - 1 + i
+    T* sgx = stx;
+    T* sgy = sty - (IN == kInGrad && g == 0 ? A.W : 0);  // (there is no row -1; it is not read)
+    if (!whole) {
+      const int r0 = g * RW, nx = rows_x(r0);
+      int xt = 0, yt = 0;
+      if (nx > 0) {
+        const Run<T> q = run_x(field, r0, nx);
+        sgx += q.lead;
+        xt = q.tail;
+        if (tid < xt) sgx[nx * A.W - xt + tid] = gx[field * fe + (size_t)(r0 + nx) * A.W - xt + tid];
+      }
+      if constexpr (IN == kInGrad) {
+        const Run<T> q = run_y(field, r0);
+        const int y0 = r0 > 0 ? r0 - 1 : 0, y1 = (A.H < r0 + RW) ? A.H : r0 + RW;
+        yt = q.tail;
+        if (tid < yt) sty[q.lead + (y1 - y0) * A.W - yt + tid] = gy[field * fe + (size_t)y1 * A.W - yt + tid];
+        sgy += q.lead;
+      }
+      if (xt + yt > 0) __syncthreads();  // the input's last elements are in place
+    }
     if constexpr (EDIT == kEditThreshold) {
       const float t2 = t2s[field];
       const int r0 = g * RW, nx = (A.H - r0) < RW ? (A.H - r0) : RW;
@@ -784,6 +873,12 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
       // 16-byte multiples, so 16 bytes (VE pixels) at a time
       constexpr int VE = 16 / (int)sizeof(T);
       const int wv = A.W / VE;
+      if (A.W % VE != 0) {  // rows at odd remainders: one pixel at a time
+        for (int idx = tid; idx < nx * A.W; idx += S::THREADS) {
+          T* yp = sgy + A.W + idx;
+          if (edit_mag2(f_to_f(sgx[idx]), f_to_f(*yp)) < t2) sgx[idx] = *yp = zero;
+        }
+      } else {
       for (int idx = tid; idx < nx * wv; idx += S::THREADS) {
         const int i = idx / wv, jv = idx - i * wv;
         uint4* xp = reinterpret_cast<uint4*>(sgx + (size_t)i * A.W) + jv;
@@ -804,6 +899,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
           *yp = yv;
         }
       }
+      }
       if (r0 > 0) {  // gy of the row above (sgy row 0)
 #pragma unroll
         for (int q = 0; q < kEdW; ++q) {
@@ -814,8 +910,8 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
       __syncthreads();
     }
     float2 v[S::R1];
-    if (ADJ && act) {
-      // z = Crop^T(grad_out): rows ia, ib at torus rows p + ia, p + ib, columns
+    if (IN != kInGrad && act) {
+      // the given Laplacian, or z = Crop^T(grad_out): rows ia, ib at torus rows p + ia, p + ib, columns
       // j < W at p + j; and the row pair's sum for the (sum grad_out) e_00 term,
       // compensated in FP32 (Knuth's TwoSum: the sum and the exact rounding
       // errors), so no FP64 work (scarce on this part) runs per value
@@ -831,10 +927,12 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
         const bool c1 = sure || (j >= 0 && j < A.W);
         const float a = (ha && c1) ? f_to_f(xa[j]) : 0.0f, b = (hb && c1) ? f_to_f(xb[j]) : 0.0f;
         v[r] = make_float2(a, b);
-        sum = two_sum_acc(sum, a, err);
-        sum = two_sum_acc(sum, b, err);
+        if constexpr (ADJ) {
+          sum = two_sum_acc(sum, a, err);
+          sum = two_sum_acc(sum, b, err);
+        }
       }
-      red[tid] = make_float2(sum, err);
+      if constexpr (ADJ) red[tid] = make_float2(sum, err);
     } else if (act) {
       const int r0 = g * RW, ia = r0 + 2 * f, ib = ia + 1;
       const bool ha = ia < A.H, hb = ib < A.H, hm = ia >= 1;  // rows present (ia - 1 < H always)
@@ -1715,9 +1813,11 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
     T* o = out + (size_t)field * A.H * A.W;
     // one stage-2 butterfly per thread: once its inputs are in registers the
     // exchange buffer is free, and the item's output rows are staged there
-    // ([2F][W], the output's own row pitch) and leave by one bulk copy
+    // ([2F][W], the output's own row pitch, at its remainder from a 16-byte
+    // boundary) and leave by one bulk copy
     const bool stage = S::J2 == 1 && A.stage_out;
-    T* srows = reinterpret_cast<T*>(buf);
+    const int r0s = g * 2 * S::F, nrs = (A.H - r0s) < 2 * S::F ? (A.H - r0s) : 2 * S::F;
+    T* srows = reinterpret_cast<T*>(buf) + (reinterpret_cast<uintptr_t>(o + (size_t)r0s * A.W) & 15) / sizeof(T);
     // STATS: this thread's stored values as float sums about its first value
     float st_sh = 0.0f, st_s = 0.0f, st_q = 0.0f;
     int st_n = 0;
@@ -1775,9 +1875,8 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
     if (stage) {
       fence_proxy_async_smem();  // the staged rows precede the bulk copy that reads them
       __syncthreads();
+      if (tid < 32) store_run(o + (size_t)r0s * A.W, srows, (unsigned)(nrs * A.W), tid);
       if (tid == 0) {
-        const int r0 = g * 2 * S::F, nr = (A.H - r0) < 2 * S::F ? (A.H - r0) : 2 * S::F;
-        bulk_store(o + (size_t)r0 * A.W, srows, (unsigned)((size_t)nr * A.W * sizeof(T)));
         bulk_store_wait_read();  // buf read out: the next item may land in it
         if (w + (int)gridDim.x < items) issue(w + gridDim.x, false);
         if (w + 2 * (int)gridDim.x < items) issue(w + 2 * gridDim.x, true);
@@ -2113,6 +2212,52 @@ static cudaError_t fast_setup(K kernel, int threads, size_t smem, int* slots) {
   return cudaSuccess;
 }
 
+// The fused row pass stages its input rows in the exchange buffers, extended
+// where the rows are longer than they are (16-byte spans of FP32 rows against 8
+// bytes of each exchange element leave short row pairs a few hundred bytes
+// over), as long as the MINB_FWD blocks an SM its registers are planned for
+// still fit: fused_smem_cap is that limit (1.5 KB of a block left for its static
+// shared memory, 1 KB reserved by the system). Measured on 24 fields of
+// 720x1080 (threshold edit): staged 86 us, through packed rows in global memory
+// 92 us.
+constexpr int kSmemPerSM = 228 * 1024, kSmemBlockMax = 227 * 1024, kSmemBlockExtra = 2560;
+template <class S>
+constexpr size_t fused_smem_cap() {
+  const size_t least = (size_t)S::R1 * S::R2 * sizeof(float2) + fused_exchange_bytes<S>();
+  size_t cap = (size_t)(kSmemPerSM / S::MINB_FWD - kSmemBlockExtra) / 16 * 16;
+  if (cap > (size_t)(kSmemBlockMax - kSmemBlockExtra)) cap = (size_t)(kSmemBlockMax - kSmemBlockExtra);
+  return cap > least ? cap : least;
+}
+// the fused row pass's shared memory for rows of W, 0 where they are too wide
+template <class S, typename T>
+static size_t fused_smem(int W, int in) {
+  const size_t st = fused_stage_bytes<S, T>(W, in), ex = fused_exchange_bytes<S>();
+  const size_t n = (size_t)S::R1 * S::R2 * sizeof(float2) + (st > ex ? st : ex);
+  return n <= fused_smem_cap<S>() ? n : 0;
+}
+// blocks of the fused row pass resident at once: `slots` at the exchange
+// buffers' size, fewer where its staging is larger
+template <class S>
+static int fused_slots(int slots, size_t smem) {
+  const size_t ex = (size_t)S::R1 * S::R2 * sizeof(float2) + fused_exchange_bytes<S>();
+  if (smem <= ex) return slots;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return slots;
+  const int fit = (int)(kSmemPerSM / (smem + kSmemBlockExtra));
+  const int lim = (fit < 1 ? 1 : fit) * sms;
+  return lim < slots ? lim : slots;
+}
+// fast_setup for the fused row pass: occupancy at the exchange buffers' size,
+// the shared-memory cap at its limit
+template <class S, typename K>
+static cudaError_t fused_setup(K kernel, int* slots) {
+  const cudaError_t e = fast_setup(kernel, S::THREADS, S::smem_bytes_fwd(), slots);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem_cap<S>());
+}
+
 }  // namespace gfc
 
 // the one-launch solve for small tori (thread-block clusters, spectrum kept in
@@ -2128,14 +2273,13 @@ namespace gfc {
 // term) and stores S with half-band sums; one warp per field reduces the sum;
 // the carry sweep runs over the half-bands with -sum at torus row 0; the
 // adjoint's inverse row pass solves each half-band in shared memory and writes
-// grad_gx, grad_gy. Needs grad_out rows that can be bulk-copied into the
-// forward pass's staging; returns cudaErrorNotSupported otherwise.
+// grad_gx, grad_gy. Needs grad_out rows that fit the forward pass's staging;
+// returns cudaErrorNotSupported otherwise.
 template <class RS, typename T>
 static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, T* ggx, T* ggy, int nf,
                                     cudaStream_t st) {
-  if ((P->W * sizeof(T)) % 16 != 0 || (size_t)2 * RS::F * P->W * sizeof(T) > fused_exchange_bytes<RS>() ||
-      getenv("GFC_UNFUSED_DIV") != nullptr)
-    return cudaErrorNotSupported;
+  const size_t smem_a = fused_smem<RS, T>(P->W, kInAdj);
+  if (smem_a == 0 || getenv("GFC_UNFUSED_DIV") != nullptr) return cudaErrorNotSupported;
   FastArgs A;
   A.stage_out = 0;
   A.invM = 1.0 / (double)P->M;
@@ -2168,9 +2312,7 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
     static bool ready = false;
     if (!ready) {
       int unused = 0;
-      if ((e = fast_setup(k_fast_rows_fwd_div<RS, T, true, true>, RS::THREADS, RS::smem_bytes_fwd(), &slots_a)) !=
-          cudaSuccess)
-        return e;
+      if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, kInAdj, true>, &slots_a)) != cudaSuccess) return e;
       if ((e = fast_setup(k_fast_rows_adj<RS, T, true>, RS::THREADS, RS::smem_bytes_adj_tri(), &slots_c)) !=
           cudaSuccess)
         return e;
@@ -2183,9 +2325,9 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   const bool one = P->block_items;
   auto grid_for = [one](long items, int slots) { return (int)((one || items < slots) ? items : slots); };
   prof_begin(P, 0, st);
-  k_fast_rows_fwd_div<RS, T, true, true><<<grid_for((long)nf * A.ngroups, slots_a), RS::THREADS,
-                                           RS::smem_bytes_fwd(), st>>>(gout, nullptr, bf.spec, P->twN, bf.partial, A,
-                                                                       bf.tri, P->colcoef_h);
+  k_fast_rows_fwd_div<RS, T, kInAdj, true>
+      <<<grid_for((long)nf * A.ngroups, fused_slots<RS>(slots_a, smem_a)), RS::THREADS, smem_a, st>>>(
+          gout, nullptr, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef_h);
   prof_end(P, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
@@ -2281,9 +2423,8 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
         }
         if ((e = fast_setup(k_fast_rows_fwd<RS, false>, RS::THREADS, RS::smem_bytes_fwd(), &slots_a)) != cudaSuccess)
           return e;
-        if (MODE != 1 && (e = fast_setup(k_fast_rows_fwd_div<RS, T, MODE == 2, false>, RS::THREADS,
-                                         RS::smem_bytes_fwd(), &slots_d)) != cudaSuccess)
-          return e;
+        if constexpr (MODE != 1)
+          if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, MODE, false>, &slots_d)) != cudaSuccess) return e;
       }
       if constexpr (MODE != 2) {
         int unused_k = 0;
@@ -2295,16 +2436,13 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
           return e;
         if ((e = fast_setup(k_fast_rows_fwd<RS, true>, RS::THREADS, RS::smem_bytes_fwd(), &slots_ta)) != cudaSuccess)
           return e;
+        if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, MODE, true>, &slots_td)) != cudaSuccess) return e;
       }
       if constexpr (MODE == 0) {
         if ((e = fast_setup(k_fast_rows_inv<RS, T, true, true>, RS::THREADS, RS::smem_bytes_tri_inv(), &slots_ts)) !=
             cudaSuccess)
           return e;
-        if ((e = fast_setup(k_fast_rows_fwd_div<RS, T, false, true>, RS::THREADS, RS::smem_bytes_fwd(), &slots_td)) !=
-            cudaSuccess)
-          return e;
-        if ((e = fast_setup(k_fast_rows_fwd_div<RS, T, false, true, kEditThreshold>, RS::THREADS,
-                            RS::smem_bytes_fwd(), &slots_tde)) != cudaSuccess)
+        if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, kInGrad, true, kEditThreshold>, &slots_tde)) != cudaSuccess)
           return e;
       }
       ready = true;
@@ -2313,32 +2451,37 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   // persistent grids (as many blocks as fit, each looping over items), or one block per item
   const bool one = P->block_items;
   auto grid_for = [one](long items, int slots) { return (int)((one || items < slots) ? items : slots); };
-  // Plain gradient solves fold pass L into the row pass, and the adjoint folds
-  // its packing of grad_out (with the row-pair sums) into it, when the rows can
-  // be bulk-copied and their staging fits the exchange buffers.
-  const size_t stage = (MODE == 2) ? (size_t)2 * RS::F * P->W * sizeof(T) : fused_stage_bytes<RS, T>(P->W);
+  // Plain gradient solves, Laplacian solves and the adjoint fold pass L (the
+  // adjoint: its packing of grad_out with the row-pair sums) into the row pass
+  // when the staged rows fit its shared memory.
+  const size_t smem_f = fused_smem<RS, T>(P->W, MODE);
   const int edit_kind = (MODE == 0 && ed) ? ed->kind : kEditNone;
   // the threshold edit is staged with the gradient (recursive column solve plans)
   const bool fused_edit = edit_kind == kEditThreshold && tri;
-  const bool fused_div = MODE != 1 && (edit_kind == kEditNone || fused_edit) && (P->W * sizeof(T)) % 16 == 0 &&
-                         stage <= fused_exchange_bytes<RS>() && getenv("GFC_UNFUSED_DIV") == nullptr;
+  const bool fused_div = (MODE != 1 || tri) && (edit_kind == kEditNone || fused_edit) && smem_f != 0 &&
+                         getenv("GFC_UNFUSED_DIV") == nullptr;
   const long a_items = (long)nf * A.ngroups;
   if (fused_div) {
     prof_begin(P, 0, st);
-    if constexpr (MODE == 0) {
-      if (fused_edit)
-        k_fast_rows_fwd_div<RS, T, false, true, kEditThreshold>
-            <<<grid_for(a_items, slots_tde), RS::THREADS, RS::smem_bytes_fwd(), st>>>(
-                in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef, ed->t2);
-      else if (tri)
-        k_fast_rows_fwd_div<RS, T, false, true><<<grid_for(a_items, slots_td), RS::THREADS, RS::smem_bytes_fwd(), st>>>(
-            in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef);
-      else if constexpr (kCols)
-        k_fast_rows_fwd_div<RS, T, false, false><<<grid_for(a_items, slots_d), RS::THREADS, RS::smem_bytes_fwd(), st>>>(
-            in0, in1, bf.spec, P->twN, bf.partial, A, nullptr, nullptr);
+    if constexpr (MODE != 2) {
+      if (fused_edit) {
+        if constexpr (MODE == 0)
+          k_fast_rows_fwd_div<RS, T, kInGrad, true, kEditThreshold>
+              <<<grid_for(a_items, fused_slots<RS>(slots_tde, smem_f)), RS::THREADS, smem_f, st>>>(
+                  in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef, ed->t2);
+      } else if (tri) {
+        k_fast_rows_fwd_div<RS, T, MODE, true>
+            <<<grid_for(a_items, fused_slots<RS>(slots_td, smem_f)), RS::THREADS, smem_f, st>>>(
+                in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef);
+      } else if constexpr (kCols && MODE == 0) {
+        k_fast_rows_fwd_div<RS, T, kInGrad, false>
+            <<<grid_for(a_items, fused_slots<RS>(slots_d, smem_f)), RS::THREADS, smem_f, st>>>(
+                in0, in1, bf.spec, P->twN, bf.partial, A, nullptr, nullptr);
+      }
     } else if constexpr (kCols) {
-      k_fast_rows_fwd_div<RS, T, MODE == 2, false><<<grid_for(a_items, slots_d), RS::THREADS, RS::smem_bytes_fwd(), st>>>(
-          in0, in1, bf.spec, P->twN, bf.partial, A, nullptr, nullptr);
+      k_fast_rows_fwd_div<RS, T, kInAdj, false>
+          <<<grid_for(a_items, fused_slots<RS>(slots_d, smem_f)), RS::THREADS, smem_f, st>>>(
+              in0, in1, bf.spec, P->twN, bf.partial, A, nullptr, nullptr);
     }
     prof_end(P, st);
   }
@@ -2393,9 +2536,8 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   FastArgs C = A;
   // the inverse row pass stages its output rows in its exchange buffer and
-  // stores them by bulk copy when the rows are whole 16-byte multiples
-  C.stage_out = MODE != 2 && (P->W * sizeof(T)) % 16 == 0 && (reinterpret_cast<uintptr_t>(out0) & 15) == 0 &&
-                (size_t)2 * RS::F * P->W * sizeof(T) <= (size_t)RS::F * RS::NP * sizeof(float2);
+  // stores them by bulk copy
+  C.stage_out = MODE != 2 && run_bytes<T>((size_t)2 * RS::F * P->W) <= (size_t)RS::F * RS::NP * sizeof(float2);
   prof_begin(P, 2, st);
   if constexpr (MODE == 2) {
     C.ngroups = (P->H + RS::F - 1) / RS::F;
