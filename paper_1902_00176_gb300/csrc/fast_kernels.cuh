@@ -2359,8 +2359,14 @@ template <class RS, class CS, typename T, int MODE>
 static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, const T* in1, T* out0, T* out1, int nf,
                                  cudaStream_t st, const EditArgs* ed = nullptr) {
   constexpr bool kCols = !std::is_same_v<CS, NoCols>;  // column transforms compiled for this shape
+  // the short lengths and 16-bit storage on the lengths compiled for their rows
+  // only: edits go through pass L and there are no statistics (fast_rows_lean);
+  // in 16 bits Laplacians go through pass L too and nothing is solved in one
+  // launch (half the kernels of a length, of two types)
+  constexpr bool kLean16 = !kCols && sizeof(T) == 2;
+  constexpr bool kLean = !kCols && (sizeof(T) == 2 || RS::N <= kRowPolicyMin);
   static_assert(!kCols || RS::N <= 2048, "the adjoint packing pass covers a whole row in one block");
-  if constexpr (MODE == 0) {
+  if constexpr (MODE == 0 && !kLean16) {
     if (P->tri && ed == nullptr) {  // plain solves of fields whose spectrum fits a cluster's shared memory
       const cudaError_t ef = run_fused_small<RS, T>(P, in0, in1, out0, nf, st);
       if (ef != cudaErrorNotSupported) return ef;
@@ -2370,6 +2376,8 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
     if (P->tri) {  // the adjoint by the recursive column solve where its staging fits
       const cudaError_t ea = run_fast_adj_tri<RS, T>(P, bf, in0, out0, out1, nf, st);
       if (ea != cudaErrorNotSupported || !kCols) return ea;
+      if constexpr (kCols)
+        if (P->M != CS::M) return ea;  // the row passes of this shape alone
     }
   }
   constexpr bool kTriMode = MODE != 2;
@@ -2436,9 +2444,10 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
           return e;
         if ((e = fast_setup(k_fast_rows_fwd<RS, true>, RS::THREADS, RS::smem_bytes_fwd(), &slots_ta)) != cudaSuccess)
           return e;
-        if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, MODE, true>, &slots_td)) != cudaSuccess) return e;
+        if constexpr (MODE == 0 || !kLean16)
+          if ((e = fused_setup<RS>(k_fast_rows_fwd_div<RS, T, MODE, true>, &slots_td)) != cudaSuccess) return e;
       }
-      if constexpr (MODE == 0) {
+      if constexpr (MODE == 0 && !kLean) {
         if ((e = fast_setup(k_fast_rows_inv<RS, T, true, true>, RS::THREADS, RS::smem_bytes_tri_inv(), &slots_ts)) !=
             cudaSuccess)
           return e;
@@ -2457,22 +2466,23 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   const size_t smem_f = fused_smem<RS, T>(P->W, MODE);
   const int edit_kind = (MODE == 0 && ed) ? ed->kind : kEditNone;
   // the threshold edit is staged with the gradient (recursive column solve plans)
-  const bool fused_edit = edit_kind == kEditThreshold && tri;
-  const bool fused_div = (MODE != 1 || tri) && (edit_kind == kEditNone || fused_edit) && smem_f != 0 &&
+  const bool fused_edit = edit_kind == kEditThreshold && tri && !kLean;
+  const bool fused_div = (MODE != 1 || (tri && !kLean16)) && (edit_kind == kEditNone || fused_edit) && smem_f != 0 &&
                          getenv("GFC_UNFUSED_DIV") == nullptr;
   const long a_items = (long)nf * A.ngroups;
   if (fused_div) {
     prof_begin(P, 0, st);
     if constexpr (MODE != 2) {
       if (fused_edit) {
-        if constexpr (MODE == 0)
+        if constexpr (MODE == 0 && !kLean)
           k_fast_rows_fwd_div<RS, T, kInGrad, true, kEditThreshold>
               <<<grid_for(a_items, fused_slots<RS>(slots_tde, smem_f)), RS::THREADS, smem_f, st>>>(
                   in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef, ed->t2);
       } else if (tri) {
-        k_fast_rows_fwd_div<RS, T, MODE, true>
-            <<<grid_for(a_items, fused_slots<RS>(slots_td, smem_f)), RS::THREADS, smem_f, st>>>(
-                in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef);
+        if constexpr (MODE == 0 || !kLean16)
+          k_fast_rows_fwd_div<RS, T, MODE, true>
+              <<<grid_for(a_items, fused_slots<RS>(slots_td, smem_f)), RS::THREADS, smem_f, st>>>(
+                  in0, in1, bf.spec, P->twN, bf.partial, A, bf.tri, P->colcoef);
       } else if constexpr (kCols && MODE == 0) {
         k_fast_rows_fwd_div<RS, T, kInGrad, false>
             <<<grid_for(a_items, fused_slots<RS>(slots_d, smem_f)), RS::THREADS, smem_f, st>>>(
@@ -2546,13 +2556,14 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   } else {
     (void)out1;
     C.ngroups = ((P->H + 1) / 2 + RS::F - 1) / RS::F;
-    const bool stats = MODE == 0 && tri && ed && ed->ref_mean;
+    const bool stats = MODE == 0 && !kLean && tri && ed && ed->ref_mean;
     if (stats && (kStatsOff + 3 * C.ngroups > kColorCoef / 2 || nkb > kStatsOff)) return cudaErrorInvalidConfiguration;
     if (stats) {
       C.nparts = nkb;
-      k_fast_rows_inv<RS, T, true, true>
-          <<<grid_for((long)nf * C.ngroups, slots_ts), RS::THREADS, RS::smem_bytes_tri_inv(), st>>>(
-              bf.spec, bf.partial, out0, P->twN, C, bf.tri, P->colcoef);
+      if constexpr (MODE == 0 && !kLean)
+        k_fast_rows_inv<RS, T, true, true>
+            <<<grid_for((long)nf * C.ngroups, slots_ts), RS::THREADS, RS::smem_bytes_tri_inv(), st>>>(
+                bf.spec, bf.partial, out0, P->twN, C, bf.tri, P->colcoef);
     } else if (tri) {
       C.nparts = nkb;
       k_fast_rows_inv<RS, T, true, false>
@@ -2584,19 +2595,19 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
 }
 
 // Shapes compiled for their row length only (the recursive column solve needs
-// no column kernels): FP32 solves and edited solves; the caller falls back to
-// the generic passes for anything else (cudaErrorNotSupported).
-template <class RS>
+// no column kernels); the caller falls back to the generic passes for anything
+// else (cudaErrorNotSupported).
+template <class RS, typename T>
 cudaError_t run_rows_shape(gfc_plan* P, const Bufs& bf, int mode, const void* in0, const void* in1, void* out0,
                            void* out1, int nf, cudaStream_t st, const EditArgs* ed) {
-  if (P->dtype != GFC_F32 || !P->tri) return cudaErrorNotSupported;
-  const float* a = static_cast<const float*>(in0);
-  const float* b = static_cast<const float*>(in1);
-  float* o0 = static_cast<float*>(out0);
-  float* o1 = static_cast<float*>(out1);
-  if (mode == 0) return run_fast_mode<RS, NoCols, float, 0>(P, bf, a, b, o0, o1, nf, st, ed);
-  if (mode == 2) return run_fast_mode<RS, NoCols, float, 2>(P, bf, a, b, o0, o1, nf, st);
-  return run_fast_mode<RS, NoCols, float, 1>(P, bf, a, b, o0, o1, nf, st);
+  if (!P->tri) return cudaErrorNotSupported;
+  const T* a = static_cast<const T*>(in0);
+  const T* b = static_cast<const T*>(in1);
+  T* o0 = static_cast<T*>(out0);
+  T* o1 = static_cast<T*>(out1);
+  if (mode == 0) return run_fast_mode<RS, NoCols, T, 0>(P, bf, a, b, o0, o1, nf, st, ed);
+  if (mode == 2) return run_fast_mode<RS, NoCols, T, 2>(P, bf, a, b, o0, o1, nf, st);
+  return run_fast_mode<RS, NoCols, T, 1>(P, bf, a, b, o0, o1, nf, st);
 }
 
 template <class RS, class CS>

@@ -187,7 +187,10 @@ cudaError_t build_colcoef(float* cc, float* pw, int M, int N, int Nh, int ldY, i
 
 // register-resident passes (solve_fast.cu): spectrum laid out [l][r]
 bool fast_supported(int M, int N);      // row and column passes compiled for M x N
-bool fast_rows_supported(int N);        // row passes compiled for N alone (recursive column solve, FP32)
+bool fast_rows_supported(int N);        // row passes compiled for N, any M (recursive column solve)
+// plans on the short lengths, and 16-bit plans, compiled without column passes: no
+// statistics in the inverse row pass (gfc_solve_corrected runs them as separate passes)
+bool fast_rows_lean(int M, int N, gfc_dtype dtype);
 int fast_row_lengths(int* out, int cap);  // compiled row lengths, ascending; returns the count
 size_t fast_zbuf_elems(int H, int M, int N);  // per field
 int fast_row_items(int M, int N);             // row pairs per item of the row passes (F)

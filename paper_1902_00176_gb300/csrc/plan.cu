@@ -284,8 +284,8 @@ gfc_status gfc_plan_create_ex(gfc_plan** out, const gfc_plan_opts* o) {
   }
   const bool usable = !p->exact && pad == 4 && getenv("GFC_FORCE_GENERIC") == nullptr;
   p->fast_cols = usable && fast_supported(M, N);
-  // row-only lengths run FP32 with the recursive column solve
-  const bool rows_only = usable && !p->fast_cols && fast_rows_supported(N) && o->dtype == GFC_F32 &&
+  // row-only lengths run with the recursive column solve
+  const bool rows_only = usable && !p->fast_cols && fast_rows_supported(N) &&
                          o->column_solver == GFC_COLUMN_RECURSIVE;
   p->fast = p->fast_cols || rows_only;
   p->tri = p->fast && o->column_solver == GFC_COLUMN_RECURSIVE;
@@ -522,7 +522,7 @@ static gfc_status create_ragged_generic(gfc_plan** out, int n, const gfc_item* i
   return GFC_OK;
 }
 
-// Ragged plans: FP32 items whose padded size has register-resident row passes
+// Ragged plans: items whose padded size has register-resident row passes
 // run as uniform sub-plans (batch 1, the item's C) on internal streams; the
 // others go through the generic per-field passes.
 static gfc_status attach_subplans(gfc_plan* p, const std::vector<int>& fast_items, const gfc_item* items) {
@@ -539,7 +539,7 @@ static gfc_status attach_subplans(gfc_plan* p, const std::vector<int>& fast_item
     const gfc_item& it = items[fast_items[j]];
     gfc_plan_opts o;
     memset(&o, 0, sizeof(o));
-    o.H = it.H; o.W = it.W; o.C = it.C; o.batch = 1; o.dtype = GFC_F32; o.pad = 4; o.streams = 1;
+    o.H = it.H; o.W = it.W; o.C = it.C; o.batch = 1; o.dtype = p->dtype; o.pad = 4; o.streams = 1;
     gfc_status st = gfc_plan_create_ex(&p->sub[j], &o);
     if (st != GFC_OK) return st;
     p->nsub = j + 1;
@@ -570,8 +570,9 @@ gfc_status gfc_plan_create_ragged(gfc_plan** out, int n, const gfc_item* items, 
     maxM = std::max(maxM, M); maxN = std::max(maxN, N); maxH = std::max(maxH, it.H); maxW = std::max(maxW, it.W);
     nfields += it.C;
     rag_total = std::max(rag_total, it.offset + (long long)it.C * it.H * it.W);
-    const bool fast = dtype == GFC_F32 && getenv("GFC_FORCE_GENERIC") == nullptr &&
-                      (fast_supported(M, N) || fast_rows_supported(N));
+    // (the sub-plans' entry points take 16-byte aligned fields)
+    const bool fast = getenv("GFC_FORCE_GENERIC") == nullptr && fast_rows_supported(N) &&
+                      it.offset * (long long)dtype_size(dtype) % 16 == 0;
     if (fast) fast_items.push_back(i);
     else generic_items.push_back(i);
   }

@@ -1,0 +1,9 @@
+// rows_family16_a.cu -- register-resident row passes in 16 bits for row lengths
+// 140 160 180 200 224 (recursive column solve only).
+#include "rows_family.cuh"
+
+namespace gfc {
+
+GFC_ROWS_A(GFC_ROW_SHAPE16)
+
+}  // namespace gfc

@@ -1,0 +1,9 @@
+// rows_family16_b.cu -- register-resident row passes in 16 bits for row lengths
+// 252 294 320 360 400 (recursive column solve only).
+#include "rows_family.cuh"
+
+namespace gfc {
+
+GFC_ROWS_B(GFC_ROW_SHAPE16)
+
+}  // namespace gfc

@@ -1,12 +1,9 @@
-// rows_family_f.cu -- register-resident row passes for row lengths 1536 1750 1960 2058
-// (schedules N = R1 x R2, F transforms per block; recursive column solve only).
+// rows_family_f.cu -- register-resident row passes in FP32 for row lengths
+// 1536 1750 1960 2058 (recursive column solve only).
 #include "rows_family.cuh"
 
 namespace gfc {
 
-GFC_ROW_SHAPE(1536,32,48,3)
-GFC_ROW_SHAPE(1750,35,50,3)
-GFC_ROW_SHAPE(1960,35,56,2)
-GFC_ROW_SHAPE(2058,42,49,2)
+GFC_ROWS_F(GFC_ROW_SHAPE)
 
 }  // namespace gfc

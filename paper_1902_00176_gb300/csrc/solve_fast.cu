@@ -15,13 +15,17 @@ GFC_FAST_SHAPE(270, 270)
 GFC_FAST_SHAPE(72, 108)
 #undef GFC_FAST_SHAPE
 
-// row lengths compiled on their own (rows_family_*.cu)
+// row lengths compiled on their own (rows_family_*.cu, rows_family16_*.cu)
 #define GFC_ROW_LEN(N)                                                                                         \
   cudaError_t fast_rows_run_##N(gfc_plan*, const Bufs&, int, const void*, const void*, void*, void*, int,     \
                                 cudaStream_t, const EditArgs*);                                               \
+  cudaError_t fast_rows_run16_##N(gfc_plan*, const Bufs&, int, const void*, const void*, void*, void*, int,   \
+                                  cudaStream_t, const EditArgs*);                                             \
   size_t fast_rows_zbuf_##N(int H);                                                                            \
   int fast_rows_items_##N();
 #define GFC_ROW_LENS(X)                                                                                          \
+  X(32) X(36) X(40) X(42) X(48) X(50) X(54) X(56) X(60) X(64) X(70) X(72) X(80) X(84) X(90) X(96) X(98) X(100)   \
+  X(112) X(120) X(126) X(128)                                                                                    \
   X(140) X(160) X(180) X(200) X(224) X(252) X(294) X(320) X(360) X(400) X(448) X(500) X(560) X(630) X(700)     \
   X(784) X(882) X(980) X(1080) X(1120) X(1200) X(1372) X(1400) X(1536) X(1750) X(1960) X(2058)
 GFC_ROW_LENS(GFC_ROW_LEN)
@@ -46,14 +50,23 @@ const FastEntry* find(int M, int N) {
     if (e.M == M && e.N == N) return &e;
   return nullptr;
 }
+// the row passes of a size pair serve its row length with any column length too
+// (recursive column solve)
+const FastEntry* find_by_rows(int N) {
+  for (const FastEntry& e : kFast)
+    if (e.N == N) return &e;
+  return nullptr;
+}
 struct RowEntry {
   int N;
   cudaError_t (*run)(gfc_plan*, const Bufs&, int, const void*, const void*, void*, void*, int, cudaStream_t,
                      const EditArgs*);
+  cudaError_t (*run16)(gfc_plan*, const Bufs&, int, const void*, const void*, void*, void*, int, cudaStream_t,
+                       const EditArgs*);
   size_t (*zbuf)(int H);
   int (*items)();
 };
-#define GFC_ROW_ENTRY(N) {N, fast_rows_run_##N, fast_rows_zbuf_##N, fast_rows_items_##N},
+#define GFC_ROW_ENTRY(N) {N, fast_rows_run_##N, fast_rows_run16_##N, fast_rows_zbuf_##N, fast_rows_items_##N},
 const RowEntry kRows[] = {GFC_ROW_LENS(GFC_ROW_ENTRY)};
 #undef GFC_ROW_ENTRY
 const RowEntry* find_rows(int N) {
@@ -65,7 +78,11 @@ const RowEntry* find_rows(int N) {
 
 bool fast_supported(int M, int N) { return find(M, N) != nullptr; }
 
-bool fast_rows_supported(int N) { return find_rows(N) != nullptr; }
+bool fast_rows_supported(int N) { return find_rows(N) != nullptr || find_by_rows(N) != nullptr; }
+
+bool fast_rows_lean(int M, int N, gfc_dtype dtype) {
+  return (dtype != GFC_F32 || N <= kRowPolicyMin) && find(M, N) == nullptr && find_rows(N) != nullptr;
+}
 
 int fast_row_lengths(int* out, int cap) {  // the listed lengths that have a kernel set
   int m = 0;
@@ -82,19 +99,23 @@ int fast_row_lengths(int* out, int cap) {  // the listed lengths that have a ker
 size_t fast_zbuf_elems(int H, int M, int N) {
   if (const FastEntry* e = find(M, N)) return e->zbuf(H);
   if (const RowEntry* r = find_rows(N)) return r->zbuf(H);
+  if (const FastEntry* e = find_by_rows(N)) return e->zbuf(H);
   return 0;
 }
 
 int fast_row_items(int M, int N) {
   if (const FastEntry* e = find(M, N)) return e->items();
   if (const RowEntry* r = find_rows(N)) return r->items();
+  if (const FastEntry* e = find_by_rows(N)) return e->items();
   return 0;
 }
 
 cudaError_t run_chunk_fast(gfc_plan* P, const Bufs& bf, int mode, const void* in0, const void* in1, void* out0,
                            void* out1, int nf, cudaStream_t st, const EditArgs* ed) {
   if (const FastEntry* e = find(P->M, P->N)) return e->run(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
-  if (const RowEntry* r = find_rows(P->N)) return r->run(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
+  if (const RowEntry* r = find_rows(P->N))
+    return (P->dtype == GFC_F32 ? r->run : r->run16)(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
+  if (const FastEntry* e = find_by_rows(P->N)) return e->run(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
   return cudaErrorNotSupported;
 }
 
