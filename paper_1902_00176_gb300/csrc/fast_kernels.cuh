@@ -117,6 +117,10 @@ __device__ __forceinline__ float2 tri_step(float2 x, float2 y, float delta) {
   return __ffma2_rn(make_float2(-delta, -delta), y, cadd(x, y));  // packed pair arithmetic
 }
 
+// one step of the carry sweep, t <- e + T t with T = 1 - D, the same way: bands of
+// a few rows have T next to 1, and its rounding would add up over the bands
+__device__ __forceinline__ float2 tri_carry(float2 e, float2 t, float D) { return tri_step(e, t, D); }
+
 __device__ __forceinline__ float f_to_f(float x) { return x; }
 __device__ __forceinline__ float f_to_f(__half x) { return __half2float(x); }
 __device__ __forceinline__ float f_to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
@@ -1217,7 +1221,7 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
     c03 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8));
     c47 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8) + 1);
   }
-  const float a = c03.y, C = c03.z, Tb = c03.w, Tl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
+  const float a = c03.y, C = c03.z, Db = c03.w, Dl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
   const int per = (A.G + kTriSeg - 1) / kTriSeg;
   const int g0 = min(warp * per, A.G), g1 = min(g0 + per, A.G);
   // phase 1: each segment from zero carries
@@ -1226,15 +1230,15 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
     if (col_ok) {
 #pragma unroll 4
       for (int g = g0; g < g1; ++g) {
-        const float T = (g == A.G - 1) ? Tl : Tb;
+        const float D = (g == A.G - 1) ? Dl : Db;
         const float2 e = sums[(size_t)g * 2 * kTriCols];
-        t = __ffma2_rn(make_float2(T, T), t, e);
+        t = tri_carry(e, t, D);
       }
 #pragma unroll 4
       for (int g = g1 - 1; g >= g0; --g) {
-        const float T = (g == A.G - 1) ? Tl : Tb;
+        const float D = (g == A.G - 1) ? Dl : Db;
         const float2 e = sums[(size_t)g * 2 * kTriCols + kTriCols];
-        q = __ffma2_rn(make_float2(T, T), q, e);
+        q = tri_carry(e, q, D);
       }
     }
     seg_e[warp][lane] = t;
@@ -1249,7 +1253,7 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
       const int b0 = min(s2 * per, A.G), b1 = min(b0 + per, A.G);
       Ts[s2] = (b1 <= b0) ? 1.0f
                           : (b1 < A.G ? __ldg(powc + (size_t)(b1 - b0) * A.ldY + k)
-                                      : __ldg(powc + (size_t)(b1 - b0 - 1) * A.ldY + k) * Tl);
+                                      : __ldg(powc + (size_t)(b1 - b0 - 1) * A.ldY + k) * (1.0f - Dl));
     }
     auto seg_T = [&](int s2) { return Ts[s2]; };
     if (warp == 0) {
@@ -1298,18 +1302,18 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
     float2 c = seg_e[warp][lane];
 #pragma unroll 4
     for (int g = g0; g < g1; ++g) {
-      const float T = (g == A.G - 1) ? Tl : Tb;
+      const float D = (g == A.G - 1) ? Dl : Db;
       const float2 e = sums[(size_t)g * 2 * kTriCols];
       carry[(size_t)(2 * g) * A.ldY] = c;
-      c = __ffma2_rn(make_float2(T, T), c, e);
+      c = tri_carry(e, c, D);
     }
     float2 q = seg_q[warp][lane];
 #pragma unroll 4
     for (int g = g1 - 1; g >= g0; --g) {
-      const float T = (g == A.G - 1) ? Tl : Tb;
+      const float D = (g == A.G - 1) ? Dl : Db;
       const float2 e = sums[(size_t)g * 2 * kTriCols + kTriCols];
       carry[(size_t)(2 * g + 1) * A.ldY] = q;
-      q = __ffma2_rn(make_float2(T, T), q, e);
+      q = tri_carry(e, q, D);
     }
   }
   if (warp == 0 && !A.adj) {  // u[0,0] (the adjoint has no offset)
@@ -1377,7 +1381,7 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
   if (col_ok) {
     const float4 c03 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8));
     const float4 c47 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8) + 1);
-    const float a = c03.y, C = c03.z, Tb = c03.w, Tl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
+    const float a = c03.y, C = c03.z, Db = c03.w, Dl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
     float2 yl, y0;
     {  // causal: the band sums in registers, from a zero carry, close the cycle, carries out
       float2 e[kTriRegG];
@@ -1388,8 +1392,8 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
 #pragma unroll
       for (int g = 0; g < kTriRegG; ++g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
-          t = __ffma2_rn(make_float2(T, T), t, e[g]);
+          const float D = (g == G - 1) ? Dl : Db;
+          t = tri_carry(e[g], t, D);
         }
       yl = make_float2(Tt * t.x * inv, Tt * t.y * inv);  // y[M-1]
       float2 c = make_float2(Tp * yl.x, Tp * yl.y);     // carry into band 0
@@ -1397,9 +1401,9 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
 #pragma unroll
       for (int g = 0; g < kTriRegG; ++g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
+          const float D = (g == G - 1) ? Dl : Db;
           carry[(size_t)(2 * g) * A.ldY] = c;
-          c = __ffma2_rn(make_float2(T, T), c, e[g]);
+          c = tri_carry(e[g], c, D);
         }
     }
     {  // anticausal, the same way up the bands
@@ -1411,8 +1415,8 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
 #pragma unroll
       for (int g = kTriRegG - 1; g >= 0; --g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
-          q = __ffma2_rn(make_float2(T, T), q, ep[g]);
+          const float D = (g == G - 1) ? Dl : Db;
+          q = tri_carry(ep[g], q, D);
         }
       y0 = make_float2(Tp * q.x * inv, Tp * q.y * inv);  // y'[0]
       if (A.adj) y0.x = (Tp * q.x - sadj) * inv;
@@ -1420,9 +1424,9 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
 #pragma unroll
       for (int g = kTriRegG - 1; g >= 0; --g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
+          const float D = (g == G - 1) ? Dl : Db;
           carry[(size_t)(2 * g + 1) * A.ldY] = c;
-          c = __ffma2_rn(make_float2(T, T), c, ep[g]);
+          c = tri_carry(ep[g], c, D);
         }
     }
     acc = (2 * k == A.N ? 1.0 : 2.0) * (double)(C * fmaf(a, yl.x, y0.x));

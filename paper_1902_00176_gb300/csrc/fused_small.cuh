@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(S::THREADS, 2) k_fused_small(const T* __restri
     if (col_ok) {
       const float4 c03 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8));
       const float4 c47 = __ldg(reinterpret_cast<const float4*>(cc + (size_t)k * 8) + 1);
-      const float a = c03.y, C = c03.z, Tb = c03.w, Tl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
+      const float a = c03.y, C = c03.z, Db = c03.w, Dl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
       // every band's sums in registers (one round of loads from the CTAs that
       // own them), then the sweep kernel's recurrences
       float2 e[kTriRegG], ep[kTriRegG];
@@ -260,33 +260,33 @@ __global__ void __launch_bounds__(S::THREADS, 2) k_fused_small(const T* __restri
 #pragma unroll
       for (int g = 0; g < kTriRegG; ++g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
-          tt = __ffma2_rn(make_float2(T, T), tt, e[g]);
+          const float D = (g == G - 1) ? Dl : Db;
+          tt = tri_carry(e[g], tt, D);
         }
       const float2 yl = make_float2(Tt * tt.x * inv, Tt * tt.y * inv);  // y[M-1]
       float2 cin = make_float2(Tp * yl.x, Tp * yl.y);                   // carry into band 0
 #pragma unroll
       for (int g = 0; g < kTriRegG; ++g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
+          const float D = (g == G - 1) ? Dl : Db;
           if (g >= gb0 && g < gb1) car[(size_t)(2 * (g - gb0)) * LDY + k] = cin;
-          cin = __ffma2_rn(make_float2(T, T), cin, e[g]);
+          cin = tri_carry(e[g], cin, D);
         }
       float2 q = make_float2(0.0f, 0.0f);
 #pragma unroll
       for (int g = kTriRegG - 1; g >= 0; --g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
-          q = __ffma2_rn(make_float2(T, T), q, ep[g]);
+          const float D = (g == G - 1) ? Dl : Db;
+          q = tri_carry(ep[g], q, D);
         }
       const float2 y0 = make_float2(Tp * q.x * inv, Tp * q.y * inv);  // y'[0]
       float2 cbl = make_float2(Tt * y0.x, Tt * y0.y);                 // carry from below the last band
 #pragma unroll
       for (int g = kTriRegG - 1; g >= 0; --g)
         if (g < G) {
-          const float T = (g == G - 1) ? Tl : Tb;
+          const float D = (g == G - 1) ? Dl : Db;
           if (g >= gb0 && g < gb1) car[(size_t)(2 * (g - gb0) + 1) * LDY + k] = cbl;
-          cbl = __ffma2_rn(make_float2(T, T), cbl, ep[g]);
+          cbl = tri_carry(ep[g], cbl, D);
         }
       // this column's share of u[0,0] = sum_l w_l U[0][l] (row 0 lies in the pad)
       acc = (2 * k == A.N ? 1.0 : 2.0) * (double)(C * fmaf(a, yl.x, y0.x));

@@ -187,13 +187,18 @@ cudaError_t build_colcoef(float* cc, float* pw, int M, int N, int Nh, int ldY, i
 
 // register-resident passes (solve_fast.cu): spectrum laid out [l][r]
 bool fast_supported(int M, int N);      // row and column passes compiled for M x N
-bool fast_rows_supported(int N);        // row passes compiled for N, any M (recursive column solve)
-// plans on the short lengths, and 16-bit plans, compiled without column passes: no
+bool fast_rows_supported(int M, int N);  // row passes for N with the recursive column solve (of length M)
+// plans on the short and the long lengths, and 16-bit plans, compiled without column passes: no
 // statistics in the inverse row pass (gfc_solve_corrected runs them as separate passes)
 bool fast_rows_lean(int M, int N, gfc_dtype dtype);
 int fast_row_lengths(int* out, int cap);  // compiled row lengths, ascending; returns the count
 size_t fast_zbuf_elems(int H, int M, int N);  // per field
 int fast_row_items(int M, int N);             // row pairs per item of the row passes (F)
+// row passes of the lengths above the compiled ones (rows_long.cu)
+bool long_rows_supported(int M, int N);
+int long_rows_items();
+cudaError_t run_long_rows(gfc_plan* P, const Bufs& B, int mode, const void* in0, const void* in1, void* out0, int nf,
+                          cudaStream_t st, const EditArgs* ed);
 // mode 0 gradient, 1 Laplacian, 2 adjoint (out1 = grad_gy)
 // `ed` (mode 0 only, may be null) applies a gradient edit as the gradient is loaded
 cudaError_t run_chunk_fast(gfc_plan* P, const Bufs& B, int mode, const void* in0, const void* in1, void* out0,

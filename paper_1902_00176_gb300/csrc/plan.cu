@@ -109,7 +109,8 @@ __global__ void k_build_green_t(float* GT, int M, int N, int Nh, int ldM) {
 // `last` rows long), followed by `tail` zero rows and the `pad` zero rows that
 // close the cycle. Row l of the table: delta = 1 - a (formed without
 // cancellation, so the pole stays exact near DC), a, C = -a / ((1 - a^2) N)
-// (1/N: the unnormalised inverse row transform), a^band, a^last, a^pad,
+// (1/N: the unnormalised inverse row transform), 1 - a^band, 1 - a^last (formed
+// without cancellation too: the sweep takes a step per band), a^pad,
 // 1 / (1 - a^M), a^tail. Column 0 (b = 2, singular) is solved exactly
 // elsewhere; its row is zero.
 // After the [Nh][8] rows, `dc` holds (delta, C) of every column compactly,
@@ -131,8 +132,9 @@ __global__ void k_build_colcoef(float* cc, float* dc, int M, int N, int Nh, int 
     c[0] = (float)delta;
     c[1] = (float)a;
     c[2] = (float)(-a / (delta * (1.0 + a) * (double)N));
-    c[3] = (float)pow(a, (double)band);
-    c[4] = (float)pow(a, (double)last);
+    const double la = log1p(-delta);  // log a
+    c[3] = (float)-expm1((double)band * la);
+    c[4] = (float)-expm1((double)last * la);
     c[5] = (float)pow(a, (double)pad);
     c[6] = (float)(1.0 / (1.0 - pow(a, (double)M)));
     c[7] = (float)pow(a, (double)tail);
@@ -285,7 +287,7 @@ gfc_status gfc_plan_create_ex(gfc_plan** out, const gfc_plan_opts* o) {
   const bool usable = !p->exact && pad == 4 && getenv("GFC_FORCE_GENERIC") == nullptr;
   p->fast_cols = usable && fast_supported(M, N);
   // row-only lengths run with the recursive column solve
-  const bool rows_only = usable && !p->fast_cols && fast_rows_supported(N) &&
+  const bool rows_only = usable && !p->fast_cols && fast_rows_supported(M, N) &&
                          o->column_solver == GFC_COLUMN_RECURSIVE;
   p->fast = p->fast_cols || rows_only;
   p->tri = p->fast && o->column_solver == GFC_COLUMN_RECURSIVE;
@@ -349,7 +351,7 @@ gfc_status gfc_plan_create_ex(gfc_plan** out, const gfc_plan_opts* o) {
   cudaError_t e = cudaGetDevice(&p->device);
   if (e == cudaSuccess) e = cudaMalloc(&p->G, (size_t)M * p->Nh * sizeof(float));
   if (e == cudaSuccess && p->fast_cols) e = cudaMalloc(&p->GT, (size_t)p->Nh * p->ldM * sizeof(float));
-  if (e == cudaSuccess && p->fast) e = cudaMalloc(&p->zbuf, p->zbuf_field * chunk * nslots * sizeof(float2));
+  if (e == cudaSuccess && p->zbuf_field) e = cudaMalloc(&p->zbuf, p->zbuf_field * chunk * nslots * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&p->twN, (size_t)N * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&p->twM, (size_t)M * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&p->spec, per_field * (size_t)chunk * nslots);
@@ -571,7 +573,7 @@ gfc_status gfc_plan_create_ragged(gfc_plan** out, int n, const gfc_item* items, 
     nfields += it.C;
     rag_total = std::max(rag_total, it.offset + (long long)it.C * it.H * it.W);
     // (the sub-plans' entry points take 16-byte aligned fields)
-    const bool fast = getenv("GFC_FORCE_GENERIC") == nullptr && fast_rows_supported(N) &&
+    const bool fast = getenv("GFC_FORCE_GENERIC") == nullptr && fast_rows_supported(M, N) &&
                       it.offset * (long long)dtype_size(dtype) % 16 == 0;
     if (fast) fast_items.push_back(i);
     else generic_items.push_back(i);

@@ -78,10 +78,13 @@ const RowEntry* find_rows(int N) {
 
 bool fast_supported(int M, int N) { return find(M, N) != nullptr; }
 
-bool fast_rows_supported(int N) { return find_rows(N) != nullptr || find_by_rows(N) != nullptr; }
+bool fast_rows_supported(int M, int N) {
+  return find_rows(N) != nullptr || find_by_rows(N) != nullptr || long_rows_supported(M, N);
+}
 
 bool fast_rows_lean(int M, int N, gfc_dtype dtype) {
-  return (dtype != GFC_F32 || N <= kRowPolicyMin) && find(M, N) == nullptr && find_rows(N) != nullptr;
+  if (find(M, N) != nullptr) return false;
+  return ((dtype != GFC_F32 || N <= kRowPolicyMin) && find_rows(N) != nullptr) || long_rows_supported(M, N);
 }
 
 int fast_row_lengths(int* out, int cap) {  // the listed lengths that have a kernel set
@@ -107,6 +110,7 @@ int fast_row_items(int M, int N) {
   if (const FastEntry* e = find(M, N)) return e->items();
   if (const RowEntry* r = find_rows(N)) return r->items();
   if (const FastEntry* e = find_by_rows(N)) return e->items();
+  if (long_rows_supported(M, N)) return long_rows_items();
   return 0;
 }
 
@@ -116,6 +120,7 @@ cudaError_t run_chunk_fast(gfc_plan* P, const Bufs& bf, int mode, const void* in
   if (const RowEntry* r = find_rows(P->N))
     return (P->dtype == GFC_F32 ? r->run : r->run16)(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
   if (const FastEntry* e = find_by_rows(P->N)) return e->run(P, bf, mode, in0, in1, out0, out1, nf, st, ed);
+  if (long_rows_supported(P->M, P->N)) return run_long_rows(P, bf, mode, in0, in1, out0, nf, st, ed);
   return cudaErrorNotSupported;
 }
 
