@@ -187,6 +187,13 @@ struct RowShape {
   static constexpr int MINB_FWD = SHORT ? 4 : cx_blocks(2, 200);
   static constexpr int MINB_INV = SHORT ? 4 : cx_blocks(R2 >= 48 ? 2 : 3, 160);
   static constexpr int MINB_ADJ = SHORT ? 4 : cx_blocks(2, 200);
+  // the adjoint's column solve writes the transforms' inputs (tri_solve_half)
+  // where a block's threads have about a column each; with fewer columns than
+  // threads the work moves from all threads to those that own a column, and with
+  // several columns a thread the solve's chains grow. ps a pixel, packed against
+  // not: N = 72 12.6 / 11.4, 128 10.2 / 10.0, 180 7.2 / 7.7, 270 7.5 / 7.9,
+  // 500 6.9 / 7.3, 784 8.1 / 8.1, 1080 9.9 / 9.6, 1568 9.4 / 8.8
+  static constexpr bool PACK_ADJ = SHORT && N > kRowPolicyMin;
   // adjoint inverse row pass: twiddles, exchange, the factor table
   // 1 - exp(2 pi i l / N) for l <= N/2, then (16-byte aligned) the F + 1 rows of
   // Y an item needs, LDY complex each
@@ -1589,11 +1596,25 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) k_fast_cols(const float2*
 // in registers, so it overlaps the stage-2 transforms and the output stores.
 // ---------------------------------------------------------------------------
 // Recursive column solve, pass C side: the 2F staged rows of band g (row-major
-// spectrum S) become rows of the solved spectrum U in place. Per column l >= 1,
-// from the band's two staged carries: the causal recursion down the band and
-// the anticausal one up it, U = C_l (y + y' - X). Column 0 already holds its
-// exact solution. Rows past the torus (band rows >= nb) are left alone: they
-// are below every image row.
+// spectrum S) become the inputs of the band's F inverse transforms in place. Per
+// column l >= 1, from the band's two staged carries: the causal recursion down the
+// band and the anticausal one up it, U = C_l (y + y' - X); column 0 already holds
+// its exact solution. Of each row pair (a, b) the column's thread has both values,
+// so it forms the transform's inputs A + i B at l and, by the Hermitian extension,
+// at N - l, and leaves them in the pair's two slots of column l: row 2f the one at
+// l, row 2f + 1 the one at N - l. The transforms then read one value per input;
+// with U left in the rows they read both rows for every input, and y crossed
+// shared memory once more (six passes over the band against three; these kernels
+// are bound by shared-memory wavefronts): the inverse pass of 100 fields of
+// 801x1200 227 -> 204 us, of 2048 bf16 fields of 256x256 315 -> 281 us. Rows past
+// the torus (band rows >= nb) hold zeros and stay so.
+template <class S>
+__device__ __forceinline__ void tri_pack_pair(float2 ya, float2 yb, bool edge, float2& lo, float2& hi) {
+  if (edge) ya.y = yb.y = 0.0f;  // bins 0 and N/2 are real in a real transform
+  lo = make_float2(ya.x - yb.y, ya.y + yb.x);
+  hi = make_float2(ya.x + yb.y, yb.x - ya.y);
+}
+
 template <class S>
 __device__ __forceinline__ void tri_solve_band(float2* buf, const float2* cbuf, const float* __restrict__ cc, int g,
                                                const FastArgs& A) {
@@ -1601,68 +1622,114 @@ __device__ __forceinline__ void tri_solve_band(float2* buf, const float2* cbuf, 
   const int nb = min(RW, A.M - A.p - g * RW);
   if constexpr (S::SHORT) {
     // short rows: one column per thread (the band's RW values of a column pair
-    // would not fit the registers of four blocks per SM)
+    // would not fit the registers of four blocks per SM); y stays in registers
+    // where x and y of the band fit them, else in the column's slots
+    constexpr bool kRegs = RW <= 18;
     const float2* dcs = reinterpret_cast<const float2*>(cc + (size_t)A.Nh * 8);  // (delta, C) per column
-    for (int k = 1 + threadIdx.x; k < A.Nh; k += blockDim.x) {
+    for (int k = threadIdx.x; k < A.Nh; k += blockDim.x) {
       const float2 dc = __ldg(dcs + k);
       float2 yc = cbuf[k], ya = cbuf[S::LDY + k];
       float2* col = buf + k;
-      float2 x[RW];
+      float2 x[RW], y[kRegs ? RW : 1];
 #pragma unroll
       for (int r = 0; r < RW; ++r) x[r] = col[(size_t)r * S::LDY];
+      if (k == 0) {
 #pragma unroll
-      for (int r = 0; r < RW; ++r)
-        if (r < nb) {
-          yc = tri_step(x[r], yc, dc.x);
+        for (int f = 0; f < S::F; ++f) col[(size_t)(2 * f) * S::LDY] = make_float2(x[2 * f].x, x[2 * f + 1].x);
+        continue;
+      }
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        if (r < nb) yc = tri_step(x[r], yc, dc.x);
+        if constexpr (kRegs)
+          y[r] = yc;
+        else
           col[(size_t)r * S::LDY] = yc;
-        }
+      }
+      const bool edge = 2 * k == S::N;
 #pragma unroll
-      for (int r = RW - 1; r >= 0; --r)
-        if (r < nb) {
-          ya = tri_step(x[r], ya, dc.x);
-          col[(size_t)r * S::LDY] = cscale(csub(cadd(col[(size_t)r * S::LDY], ya), x[r]), dc.y);
+      for (int f = S::F - 1; f >= 0; --f) {
+        float2 u[2];
+#pragma unroll
+        for (int h = 1; h >= 0; --h) {
+          const int r = 2 * f + h;
+          u[h] = x[r];
+          if (r < nb) {
+            ya = tri_step(x[r], ya, dc.x);
+            u[h] = cscale(csub(cadd(kRegs ? y[kRegs ? r : 0] : col[(size_t)r * S::LDY], ya), x[r]), dc.y);
+          }
         }
+        float2 lo, hi;
+        tri_pack_pair<S>(u[0], u[1], edge, lo, hi);
+        col[(size_t)(2 * f) * S::LDY] = lo;
+        col[(size_t)(2 * f + 1) * S::LDY] = hi;
+      }
     }
   } else {
-  // thread t takes the column pair (2j, 2j + 1), 16-byte shared-memory accesses;
-  // column 0 (already solved) and columns >= Nh pass through unchanged
-  for (int j = threadIdx.x; 2 * j < A.Nh; j += blockDim.x) {
-    const int k0 = 2 * j;
-    const bool v0 = k0 >= 1, v1 = k0 + 1 < A.Nh;
-    // (delta, C) of both columns in one coalesced 16-byte load (the plan's compact table)
-    const float4 dc = __ldg(reinterpret_cast<const float4*>(cc + (size_t)A.Nh * 8) + j);
-    const float dl0 = dc.x, C0 = v0 ? dc.y : 1.0f, dl1 = dc.z, C1 = v1 ? dc.w : 1.0f;
-    const float4 yc4 = reinterpret_cast<const float4*>(cbuf)[j];
-    const float4 ya4 = reinterpret_cast<const float4*>(cbuf + S::LDY)[j];
-    float2 yc0 = make_float2(yc4.x, yc4.y), yc1 = make_float2(yc4.z, yc4.w);
-    float2 ya0 = make_float2(ya4.x, ya4.y), ya1 = make_float2(ya4.z, ya4.w);
-    float4* col = reinterpret_cast<float4*>(buf) + j;
-    float4 x[RW];
+    // thread t takes the column pair (2j, 2j + 1), 16-byte shared-memory accesses;
+    // columns >= Nh are padding
+    for (int j = threadIdx.x; 2 * j < A.Nh; j += blockDim.x) {
+      const int k0 = 2 * j;
+      // (delta, C) of both columns in one coalesced 16-byte load (the plan's compact table)
+      const float4 dc = __ldg(reinterpret_cast<const float4*>(cc + (size_t)A.Nh * 8) + j);
+      const float4 yc4 = reinterpret_cast<const float4*>(cbuf)[j];
+      const float4 ya4 = reinterpret_cast<const float4*>(cbuf + S::LDY)[j];
+      float2 yc0 = make_float2(yc4.x, yc4.y), yc1 = make_float2(yc4.z, yc4.w);
+      float2 ya0 = make_float2(ya4.x, ya4.y), ya1 = make_float2(ya4.z, ya4.w);
+      float4* col = reinterpret_cast<float4*>(buf) + j;
+      float4 x[RW], y[RW];
 #pragma unroll
-    for (int r = 0; r < RW; ++r) x[r] = col[(size_t)r * (S::LDY / 2)];
+      for (int r = 0; r < RW; ++r) x[r] = col[(size_t)r * (S::LDY / 2)];
 #pragma unroll
-    for (int r = 0; r < RW; ++r)
-      if (r < nb) {
-        yc0 = tri_step(make_float2(x[r].x, x[r].y), yc0, dl0);
-        yc1 = tri_step(make_float2(x[r].z, x[r].w), yc1, dl1);
-        col[(size_t)r * (S::LDY / 2)] = make_float4(yc0.x, yc0.y, yc1.x, yc1.y);
-      }
-#pragma unroll
-    for (int r = RW - 1; r >= 0; --r)
-      if (r < nb) {
-        ya0 = tri_step(make_float2(x[r].x, x[r].y), ya0, dl0);
-        ya1 = tri_step(make_float2(x[r].z, x[r].w), ya1, dl1);
-        const float4 y = col[(size_t)r * (S::LDY / 2)];
-        const float2 u0 = cscale(csub(cadd(make_float2(y.x, y.y), ya0), make_float2(x[r].x, x[r].y)), C0);
-        const float2 u1 = cscale(csub(cadd(make_float2(y.z, y.w), ya1), make_float2(x[r].z, x[r].w)), C1);
-        float4 u = make_float4(u0.x, u0.y, u1.x, u1.y);
-        if (!v0) {  // column 0 keeps its exact solution
-          u.x = x[r].x;
-          u.y = x[r].y;
+      for (int r = 0; r < RW; ++r) {
+        if (r < nb) {
+          yc0 = tri_step(make_float2(x[r].x, x[r].y), yc0, dc.x);
+          yc1 = tri_step(make_float2(x[r].z, x[r].w), yc1, dc.z);
         }
-        col[(size_t)r * (S::LDY / 2)] = u;
+        y[r] = make_float4(yc0.x, yc0.y, yc1.x, yc1.y);
       }
+      const bool e0 = k0 == 0 || 2 * k0 == S::N, e1 = 2 * (k0 + 1) == S::N;
+#pragma unroll
+      for (int f = S::F - 1; f >= 0; --f) {
+        float2 u0[2], u1[2];
+#pragma unroll
+        for (int h = 1; h >= 0; --h) {
+          const int r = 2 * f + h;
+          const float2 x0 = make_float2(x[r].x, x[r].y), x1 = make_float2(x[r].z, x[r].w);
+          u0[h] = x0;
+          u1[h] = x1;
+          if (r < nb) {
+            ya0 = tri_step(x0, ya0, dc.x);
+            ya1 = tri_step(x1, ya1, dc.z);
+            if (k0 > 0) u0[h] = cscale(csub(cadd(make_float2(y[r].x, y[r].y), ya0), x0), dc.y);
+            u1[h] = cscale(csub(cadd(make_float2(y[r].z, y[r].w), ya1), x1), dc.w);
+          }
+        }
+        float2 lo0, hi0, lo1, hi1;
+        tri_pack_pair<S>(u0[0], u0[1], e0, lo0, hi0);
+        tri_pack_pair<S>(u1[0], u1[1], e1, lo1, hi1);
+        col[(size_t)(2 * f) * (S::LDY / 2)] = make_float4(lo0.x, lo0.y, lo1.x, lo1.y);
+        col[(size_t)(2 * f + 1) * (S::LDY / 2)] = make_float4(hi0.x, hi0.y, hi1.x, hi1.y);
+      }
+    }
   }
+}
+
+// stage-1 inputs of transform f from the slots tri_solve_band left: input l of
+// row 2f at l below N/2, of row 2f + 1 at N - l from N/2 on
+template <class S>
+__device__ __forceinline__ void tri_load_pair(float2 (&v)[S::R1], const float2* band, int f, int t) {
+  constexpr int half = S::N / 2;
+  const float2* lo_row = band + (size_t)(2 * f) * S::LDY;
+  const float2* hi_row = lo_row + S::LDY + S::N;
+#pragma unroll
+  for (int r = 0; r < S::R1; ++r) {
+    // l = t + R2 r with t < R2: whether l lies below or above N/2 is known at
+    // compile time except for the one r whose range contains N/2
+    const int l = t + S::R2 * r;
+    const bool all_lo = S::R2 * r + S::R2 - 1 < half;
+    const bool all_hi = S::R2 * r >= half;
+    v[r] = all_lo ? lo_row[l] : (all_hi ? hi_row[-l] : *(l < half ? lo_row + l : hi_row - l));
   }
 }
 
@@ -1783,9 +1850,12 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
     }
     const int ia = g * 2 * S::F + 2 * f, ib = ia + 1;
     const bool va = act && ia < A.H, vb = act && ib < A.H;
+    float2 v[S::R1];
+    if constexpr (TRI) {
+      tri_load_pair<S>(v, buf, act ? f : 0, t);
+    } else {
     const float2* ya_row = buf + (size_t)(va ? 2 * f : 0) * A.ldY;
     const float2* yb_row = buf + (size_t)(vb ? 2 * f + 1 : 0) * A.ldY;
-    float2 v[S::R1];
 #pragma unroll
     for (int r = 0; r < S::R1; ++r) {
       // l = t + R2 r with t < R2: whether l lies below or above N/2 is known at
@@ -1804,6 +1874,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
         yb.y = 0.0f;
       }
       v[r] = lo ? make_float2(ya.x - yb.y, ya.y + yb.x) : make_float2(ya.x + yb.y, yb.x - ya.y);
+    }
     }
     if (act) dft_reg<S::R1, +1>(v);
     __syncthreads();  // every staged row read: buf becomes the exchange buffer
@@ -2002,14 +2073,64 @@ __global__ void __launch_bounds__(256) k_fast_color_apply(T* __restrict__ out, c
 // A + i B gives grad_gx in its real part and grad_gy in its imaginary part.
 // ---------------------------------------------------------------------------
 // Recursive column solve, the adjoint's inverse pass side: the F staged rows of
-// half-band g of S (and row F, the next half-band's first row) become rows of
-// the solved spectrum U in place, from the half-band's two carries, one column
-// per thread: the causal recursion down the half-band, row F from the causal
-// value above it and the anticausal carry (which is y' at row F), then the
-// anticausal recursion up, U = C_l (y + y' - X). Column 0 already holds its
-// exact solution; rows past the torus are left alone (no output row needs them).
+// half-band g of S (and row F, the next half-band's first row) become the inputs
+// of the half-band's F inverse transforms, one column per thread. From the
+// half-band's two carries: the causal recursion down the half-band, row F from the
+// causal value above it and the anticausal carry (which is y' at row F), then the
+// anticausal recursion up, U = C_l (y + y' - X); column 0 already holds its exact
+// solution. With A_i = d_l U_i (d_l = 1 - exp(2 pi i l / N)) and B_i = U_i - U_(i+1)
+// the thread writes A_i + i B_i at l and its Hermitian extension at N - l of
+// transform i's buffer, so the transforms read one value per input and the staged
+// rows are free for the next item. (Solved in place, they read U_i, U_(i+1) and d
+// for every input: five passes over the data against two and a half.) Rows past
+// the torus keep X, which is zero there: no output row needs them.
 template <class S>
-__device__ __forceinline__ void tri_solve_half(float2* stg, const float2* cbuf, const float* __restrict__ cc, int g,
+__device__ __forceinline__ void tri_solve_half(const float2* stg, const float2* cbuf, const float2* dtab, float2* buf,
+                                               const float* __restrict__ cc, int g, const FastArgs& A) {
+  constexpr int F = S::F;
+  const int nb = min(F, A.M - A.p - g * F);
+  const bool extra = nb == F && g * F + F < A.srows;
+  const float2* dcs = reinterpret_cast<const float2*>(cc + (size_t)A.Nh * 8);  // (delta, C) per column
+  for (int k = threadIdx.x; k < A.Nh; k += blockDim.x) {
+    const float2 dc = __ldg(dcs + k), d = dtab[k];
+    float2 yc = cbuf[k], ya = cbuf[S::LDY + k];
+    const float2* col = stg + k;
+    float2 x[F], y[F];
+#pragma unroll
+    for (int r = 0; r < F; ++r) x[r] = col[(size_t)r * S::LDY];
+    const bool solve = k > 0, edge = k == 0 || 2 * k == S::N;
+#pragma unroll
+    for (int r = 0; r < F; ++r) {
+      if (r < nb) yc = tri_step(x[r], yc, dc.x);
+      y[r] = yc;
+    }
+    float2 un = make_float2(0.0f, 0.0f);  // U of the row below
+    if (extra) {
+      const float2 xf = col[(size_t)F * S::LDY];
+      un = solve ? cscale(csub(cadd(tri_step(xf, yc, dc.x), ya), xf), dc.y) : xf;
+    }
+    float2* z = buf + k;
+#pragma unroll
+    for (int r = F - 1; r >= 0; --r) {
+      float2 u = x[r];
+      if (r < nb) {
+        ya = tri_step(x[r], ya, dc.x);
+        if (solve) u = cscale(csub(cadd(y[r], ya), x[r]), dc.y);
+      }
+      float2 p = u, q = un;
+      if (edge) p.y = q.y = 0.0f;  // bins 0 and N/2 are real in a real transform
+      const float2 a = cmul(p, d), b = csub(p, q);
+      if (2 * k < S::N) z[r * S::NP] = make_float2(a.x - b.y, a.y + b.x);
+      if (solve) z[r * S::NP + S::N - 2 * k] = make_float2(a.x + b.y, b.x - a.y);
+      un = u;
+    }
+  }
+}
+
+// The same with the solved rows U left in place of the staged ones (column 0 kept),
+// for transforms that read U_i and U_(i+1) themselves: see PACK_ADJ.
+template <class S>
+__device__ __forceinline__ void tri_solve_half_rows(float2* stg, const float2* cbuf, const float* __restrict__ cc, int g,
                                                const FastArgs& A) {
   constexpr int F = S::F;
   const int nb = min(F, A.M - A.p - g * F);
@@ -2111,18 +2232,34 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_ADJ) k_fast_rows_adj(const
     const int i = g * S::F + f;  // output row of this transform
     const bool vi = act && i < A.H;
     const bool landed = mbar_wait(&bar, phase);
+    float2 v[S::R1];
+    if constexpr (TRI && S::PACK_ADJ) {
+      // (the barrier also ends the previous item's stage 2 with buf)
+      if (__syncthreads_or(!landed)) {  // the copies never completed: report, let them drain, stop
+        if (tid == 0) atomicExch(A.err, kErrBulkWait);
+        mbar_wait(&bar, phase);
+        return;
+      }
+      tri_solve_half<S>(stg, cbuf, dtab, buf, cc, g, A);
+      fence_proxy_async_smem();  // this thread's reads of the staged rows precede the next bulk copy
+      __syncthreads();           // the transforms' inputs visible; the staged rows read
+      if (tid == 0 && w + (int)gridDim.x < items) issue(w + gridDim.x, false);
+      if (tid == 0 && w + 2 * (int)gridDim.x < items) issue(w + 2 * gridDim.x, true);
+#pragma unroll
+      for (int r = 0; r < S::R1; ++r) v[r] = mybuf[t + S::R2 * r];
+      __syncthreads();  // every input read: buf becomes the exchange buffer
+    } else {
     if constexpr (TRI) {
       if (__syncthreads_or(!landed)) {  // the copies never completed: report, let them drain, stop
         if (tid == 0) atomicExch(A.err, kErrBulkWait);
         mbar_wait(&bar, phase);
         return;
       }
-      tri_solve_half<S>(stg, cbuf, cc, g, A);
+      tri_solve_half_rows<S>(stg, cbuf, cc, g, A);
       __syncthreads();
     }
     const float2* y0 = stg + (size_t)(vi ? f : 0) * A.ldY;
     const float2* y1 = y0 + A.ldY;  // row i + 1 (Y holds H + 1 rows)
-    float2 v[S::R1];
 #pragma unroll
     for (int r = 0; r < S::R1; ++r) {
       const int l = t + S::R2 * r;
@@ -2150,6 +2287,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_ADJ) k_fast_rows_adj(const
     // every staged row read, and the previous item's stage 2 done with buf
     if (tid == 0 && w + (int)gridDim.x < items) issue(w + gridDim.x, false);
     if (tid == 0 && w + 2 * (int)gridDim.x < items) issue(w + 2 * gridDim.x, true);
+    }
     if (act) {
       dft_reg<S::R1, +1>(v);
 #pragma unroll

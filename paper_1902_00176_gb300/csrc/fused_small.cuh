@@ -327,7 +327,6 @@ __global__ void __launch_bounds__(S::THREADS, 2) k_fused_small(const T* __restri
   __syncthreads();
   // ---- step 3: in-band solve, inverse row transforms, offset, crop, cast
   const float u00 = u00s;
-  const int half = S::N / 2;
   T* o = out + (size_t)field * fe;
 #pragma unroll 1
   for (int g = gb0; g < gb1; ++g) {
@@ -338,27 +337,8 @@ __global__ void __launch_bounds__(S::THREADS, 2) k_fused_small(const T* __restri
     __syncthreads();  // the band's solved rows visible; the exchange is free
     const int ia = g * RW + 2 * f, ib = ia + 1;
     const bool va = act && ia < A.H, vb = act && ib < A.H;
-    const float2* ya_row = band + (size_t)(va ? 2 * f : 0) * LDY;
-    const float2* yb_row = band + (size_t)(vb ? 2 * f + 1 : 0) * LDY;
     float2 v[S::R1];
-#pragma unroll
-    for (int r = 0; r < S::R1; ++r) {
-      // Hermitian extension of the two rows' half spectra, packed into one
-      // complex transform (row ia real part, row ib imaginary part)
-      const int l = t + S::R2 * r;
-      const bool all_lo = S::R2 * r + S::R2 - 1 < half;
-      const bool all_hi = S::R2 * r > half;
-      const bool lo = all_lo || (!all_hi && l < half);
-      const int src = lo ? l : S::N - l;
-      float2 ya = va ? ya_row[src] : make_float2(0.0f, 0.0f);
-      float2 yb = vb ? yb_row[src] : make_float2(0.0f, 0.0f);
-      const bool may_edge = (r == 0) || (!all_lo && !all_hi);
-      if (may_edge && (src == 0 || src == half)) {  // bins 0 and N/2 are real
-        ya.y = 0.0f;
-        yb.y = 0.0f;
-      }
-      v[r] = lo ? make_float2(ya.x - yb.y, ya.y + yb.x) : make_float2(ya.x + yb.y, yb.x - ya.y);
-    }
+    tri_load_pair<S>(v, band, act ? f : 0, t);
     if (act) {
       dft_reg<S::R1, +1>(v);
 #pragma unroll
