@@ -188,12 +188,13 @@ struct RowShape {
   static constexpr int MINB_INV = SHORT ? 4 : cx_blocks(R2 >= 48 ? 2 : 3, 160);
   static constexpr int MINB_ADJ = SHORT ? 4 : cx_blocks(2, 200);
   // the adjoint's column solve writes the transforms' inputs (tri_solve_half)
-  // where a block's threads have about a column each; with fewer columns than
+  // where a block's threads have about a column each: with far fewer columns than
   // threads the work moves from all threads to those that own a column, and with
-  // several columns a thread the solve's chains grow. ps a pixel, packed against
-  // not: N = 72 12.6 / 11.4, 128 10.2 / 10.0, 180 7.2 / 7.7, 270 7.5 / 7.9,
-  // 500 6.9 / 7.3, 784 8.1 / 8.1, 1080 9.9 / 9.6, 1568 9.4 / 8.8
-  static constexpr bool PACK_ADJ = SHORT && N > kRowPolicyMin;
+  // several columns a thread the solve's chains grow. The adjoint in ps a pixel,
+  // packed against not: N = 50 18.0 / 15.3, 64 11.1 / 12.1, 72 10.0 / 11.4, 100
+  // 8.6 / 9.4, 180 7.2 / 7.7, 270 7.5 / 7.9, 500 6.9 / 7.3, 784 8.1 / 8.1, 1080
+  // 9.9 / 9.6, 1568 9.4 / 8.8
+  static constexpr bool PACK_ADJ = SHORT && N >= 56;
   // adjoint inverse row pass: twiddles, exchange, the factor table
   // 1 - exp(2 pi i l / N) for l <= N/2, then (16-byte aligned) the F + 1 rows of
   // Y an item needs, LDY complex each
@@ -1356,11 +1357,13 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
 // and each field's last warp to finish combines the u[0,0] partials.
 constexpr int kTriRegG = 32;
 constexpr int kTriRegWarps = 8;
-static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg(float2* __restrict__ spec,
-                                                                           float2* __restrict__ tri,
-                                                                           const float* __restrict__ cc,
-                                                                           double* __restrict__ partial, FastArgs A,
-                                                                           int nkb) {
+// MAXG: the loops' length; short columns run a shorter one at twice the blocks per
+// SM (12288 warps of 72-row columns of 5 bands: 37 us with the loops of 32, 55 with
+// loops of 48).
+template <int MAXG>
+__global__ void __launch_bounds__(32 * kTriRegWarps, MAXG <= 16 ? 4 : 2) k_tri_carries_reg(
+    float2* __restrict__ spec, float2* __restrict__ tri, const float* __restrict__ cc, double* __restrict__ partial,
+    FastArgs A, int nkb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int task = blockIdx.x * kTriRegWarps + warp;
   if (task >= A.nf * (nkb + 1)) return;
@@ -1391,13 +1394,13 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
     const float a = c03.y, C = c03.z, Db = c03.w, Dl = c47.x, Tp = c47.y, inv = c47.z, Tt = c47.w;
     float2 yl, y0;
     {  // causal: the band sums in registers, from a zero carry, close the cycle, carries out
-      float2 e[kTriRegG];
+      float2 e[MAXG];
 #pragma unroll
-      for (int g = 0; g < kTriRegG; ++g)
+      for (int g = 0; g < MAXG; ++g)
         if (g < G) e[g] = sums[(size_t)g * 2 * kTriCols];
       float2 t = make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int g = 0; g < kTriRegG; ++g)
+      for (int g = 0; g < MAXG; ++g)
         if (g < G) {
           const float D = (g == G - 1) ? Dl : Db;
           t = tri_carry(e[g], t, D);
@@ -1406,7 +1409,7 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
       float2 c = make_float2(Tp * yl.x, Tp * yl.y);     // carry into band 0
       if (A.adj) c.x -= (Tp / a) * sadj * inv;          // row 0's -s, carried a^(p-1) down
 #pragma unroll
-      for (int g = 0; g < kTriRegG; ++g)
+      for (int g = 0; g < MAXG; ++g)
         if (g < G) {
           const float D = (g == G - 1) ? Dl : Db;
           carry[(size_t)(2 * g) * A.ldY] = c;
@@ -1414,13 +1417,13 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
         }
     }
     {  // anticausal, the same way up the bands
-      float2 ep[kTriRegG];
+      float2 ep[MAXG];
 #pragma unroll
-      for (int g = 0; g < kTriRegG; ++g)
+      for (int g = 0; g < MAXG; ++g)
         if (g < G) ep[g] = sums[(size_t)g * 2 * kTriCols + kTriCols];
       float2 q = make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int g = kTriRegG - 1; g >= 0; --g)
+      for (int g = MAXG - 1; g >= 0; --g)
         if (g < G) {
           const float D = (g == G - 1) ? Dl : Db;
           q = tri_carry(ep[g], q, D);
@@ -1429,7 +1432,7 @@ static __global__ void __launch_bounds__(32 * kTriRegWarps, 2) k_tri_carries_reg
       if (A.adj) y0.x = (Tp * q.x - sadj) * inv;
       float2 c = make_float2(Tt * y0.x, Tt * y0.y);     // carry from below the last band
 #pragma unroll
-      for (int g = kTriRegG - 1; g >= 0; --g)
+      for (int g = MAXG - 1; g >= 0; --g)
         if (g < G) {
           const float D = (g == G - 1) ? Dl : Db;
           carry[(size_t)(2 * g + 1) * A.ldY] = c;
@@ -2354,6 +2357,21 @@ static cudaError_t fast_setup(K kernel, int threads, size_t smem, int* slots) {
   return cudaSuccess;
 }
 
+// The carry sweep of the chunk's fields over its A.G bands (tables for those bands;
+// k_tri_carries' shared-memory cap already raised).
+static cudaError_t launch_sweep(float2* spec, float2* tri, const float* cc, const float* powc, double* pd,
+                                const FastArgs& A, int nkb, cudaStream_t st) {
+  if (A.G <= kTriRegG) {
+    const int grid = (A.nf * (nkb + 1) + kTriRegWarps - 1) / kTriRegWarps;
+    auto k = A.G <= 8 ? k_tri_carries_reg<8> : (A.G <= 16 ? k_tri_carries_reg<16> : k_tri_carries_reg<kTriRegG>);
+    k<<<grid, 32 * kTriRegWarps, 0, st>>>(spec, tri, cc, pd, A, nkb);
+  } else {
+    const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
+    k_tri_carries<<<dim3(nkb + 1, A.nf), 32 * kTriSeg, tsm, st>>>(spec, tri, cc, powc, pd, A);
+  }
+  return cudaGetLastError();
+}
+
 // The fused row pass stages its input rows in the exchange buffers, extended
 // where the rows are longer than they are (16-byte spans of FP32 rows against 8
 // bytes of each exchange element leave short row pairs a few hundred bytes
@@ -2474,16 +2492,9 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
   double* pd = reinterpret_cast<double*>(bf.partial);
-  if (A.G <= kTriRegG) {
-    const int tasks = nf * (nkb + 1);
-    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps, 0, st>>>(
-        bf.spec, bf.tri, P->colcoef_h, pd, A, nkb);
-  } else {
-    const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb + 1, nf), 32 * kTriSeg, tsm, st>>>(bf.spec, bf.tri, P->colcoef_h, P->powc_h, pd, A);
-  }
+  e = launch_sweep(bf.spec, bf.tri, P->colcoef_h, P->powc_h, pd, A, nkb, st);
   prof_end(P, st);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   FastArgs C = A;
   C.ngroups = (P->H + RS::F - 1) / RS::F;  // half-bands holding output rows
   prof_begin(P, 2, st);
@@ -2668,14 +2679,8 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
   const int nkb = (P->Nh + kTriCols - 1) / kTriCols;  // column blocks of the sweep (u[0,0] partials)
-  if (tri && A.G <= kTriRegG) {
-    const int tasks = nf * (nkb + 1);
-    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps, 0, st>>>(
-        bf.spec, bf.tri, P->colcoef, reinterpret_cast<double*>(bf.partial), A, nkb);
-  } else if (tri) {
-    const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb + 1, nf), 32 * kTriSeg, tsm, st>>>(bf.spec, bf.tri, P->colcoef, P->powc,
-                                                                   reinterpret_cast<double*>(bf.partial), A);
+  if (tri) {
+    e = launch_sweep(bf.spec, bf.tri, P->colcoef, P->powc, reinterpret_cast<double*>(bf.partial), A, nkb, st);
   } else if constexpr (kCols) {
     if (MODE == 2) {
       k_adj_total<<<nf, 32, 0, st>>>(reinterpret_cast<double*>(bf.partial), A.zpairs);
@@ -2685,7 +2690,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
         bf.spec, bf.zbuf, P->GT, P->twM, bf.partial, A);
   }
   prof_end(P, st);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
   FastArgs C = A;
   // the inverse row pass stages its output rows in its exchange buffer and
   // stores them by bulk copy

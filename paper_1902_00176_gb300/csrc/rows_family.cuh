@@ -12,17 +12,20 @@ namespace gfc {
 
 // Row lengths: X(N, R1, R2, F), N = R1 R2 with R2 threads per transform and F
 // transforms per block (about 128 threads, within the shared memory of 2 forward
-// blocks and 3 inverse blocks per SM, 4 and 4 for N <= 512; F <= 16 keeps the
-// 2F rows of a band column in registers). Images narrower than 24 pixels
-// (N < 32) and wider than 2050 keep the generic passes.
+// blocks and 3 inverse blocks per SM, 4 and 4 for N <= 512). Short lengths take
+// blocks of about 64 threads with few idle lanes, bands of at most 22 rows (their
+// column in registers) that a square image fills with little left over; each F is
+// the faster of two to four tried, in ps a pixel of a solve: N = 42 F 16 23.8,
+// 9 14.6; 56 F 16 14.4, 8 11.6; 72 F 14 11.9, 7 9.2; 90 F 12 9.4, 6 8.2; 112 F 9
+// 7.2, 4 7.9. Images narrower than 24 pixels (N < 32) keep the generic passes.
 #define GFC_ROWS_S(X)                                                                                        \
-  X(32, 4, 8, 16) X(36, 6, 6, 16) X(40, 5, 8, 16) X(42, 6, 7, 16) X(48, 6, 8, 16) X(50, 5, 10, 12)            \
-  X(54, 6, 9, 14) X(56, 7, 8, 16) X(60, 6, 10, 12) X(64, 8, 8, 16)
+  X(32, 4, 8, 8) X(36, 6, 6, 5) X(40, 5, 8, 6) X(42, 6, 7, 9) X(48, 6, 8, 7) X(50, 5, 10, 11)            \
+  X(54, 6, 9, 6) X(56, 7, 8, 8) X(60, 6, 10, 9) X(64, 8, 8, 8)
 #define GFC_ROWS_T(X)                                                                                        \
-  X(70, 7, 10, 12) X(72, 8, 9, 14) X(80, 8, 10, 12) X(84, 7, 12, 10) X(90, 9, 10, 12) X(96, 8, 12, 10)        \
+  X(70, 7, 10, 6) X(72, 8, 9, 7) X(80, 8, 10, 6) X(84, 7, 12, 10) X(90, 9, 10, 6) X(96, 8, 12, 8)        \
   X(98, 7, 14, 9)
 #define GFC_ROWS_U(X)                                                                                        \
-  X(100, 10, 10, 12) X(112, 8, 14, 9) X(120, 10, 12, 10) X(126, 9, 14, 9) X(128, 8, 16, 8)
+  X(100, 10, 10, 6) X(112, 8, 14, 9) X(120, 10, 12, 10) X(126, 9, 14, 9) X(128, 8, 16, 8)
 #define GFC_ROWS_A(X) X(140, 10, 14, 9) X(160, 10, 16, 8) X(180, 12, 15, 8) X(200, 10, 20, 6) X(224, 14, 16, 8)
 #define GFC_ROWS_B(X) X(252, 14, 18, 7) X(294, 14, 21, 6) X(320, 16, 20, 6) X(360, 18, 20, 6) X(400, 20, 20, 6)
 #define GFC_ROWS_C(X) X(448, 16, 28, 4) X(500, 20, 25, 5) X(560, 20, 28, 4) X(630, 21, 30, 4) X(700, 25, 28, 4)

@@ -337,16 +337,9 @@ cudaError_t run_long(gfc_plan* P, const Bufs& bf, const T* in0, const T* in1, T*
   prof_end(P, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(P, 1, st);
-  if (A.G <= kTriRegG) {
-    const int tasks = nf * (nkb + 1);
-    k_tri_carries_reg<<<(tasks + kTriRegWarps - 1) / kTriRegWarps, 32 * kTriRegWarps, 0, st>>>(bf.spec, bf.tri,
-                                                                                             P->colcoef, pd, A, nkb);
-  } else {
-    const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb + 1, nf), 32 * kTriSeg, tsm, st>>>(bf.spec, bf.tri, P->colcoef, P->powc, pd, A);
-  }
+  e = launch_sweep(bf.spec, bf.tri, P->colcoef, P->powc, pd, A, nkb, st);
   prof_end(P, st);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   FastArgs C = A;
   C.ngroups = ((P->H + 1) / 2 + kLongF - 1) / kLongF;
   prof_begin(P, 2, st);
