@@ -2011,30 +2011,32 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
 // x <- (x - mean) gain + ref_mean, 16 bytes per access where the field allows.
 constexpr int kColorCoef = 1200;  // float offset (past the item statistics, 3 doubles per item)
 
-__device__ __forceinline__ void chan_d(double& n, double& m, double& m2, double nb, double mb, double m2b) {
-  const double nt = n + nb;
-  if (nt > 0.0) {
-    const double d = mb - m, fb = nb / nt;
-    m += d * fb;
-    m2 += m2b + d * d * n * fb;
-  }
-  n = nt;
-}
-
 static __global__ void __launch_bounds__(256) k_fast_color_finish(float* __restrict__ partial, int nitems, int nf,
                                                                   const float* __restrict__ ref_mean,
                                                                   const float* __restrict__ ref_std) {
   const int field = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (field >= nf) return;
   const double* pp = reinterpret_cast<const double*>(partial) + (size_t)field * (kMaxRowBlocks / 2) + kStatsOff;
-  double n = 0.0, m = 0.0, m2 = 0.0;
-  for (int i = lane; i < nitems; i += 32) chan_d(n, m, m2, pp[3 * i], pp[3 * i + 1], pp[3 * i + 2]);
+  // N = sum n_i, mean = sum n_i m_i / N, M2 = sum (M2_i + n_i (m_i - mean)^2): one
+  // FP64 division a field (pairwise updates of (n, m, M2) take one a step, 2 us each
+  // here: 19 us for 24 fields of 120 items, 4 us this way)
+  double n = 0.0, s = 0.0, m2 = 0.0;
+  for (int i = lane; i < nitems; i += 32) {
+    n += pp[3 * i];
+    s += pp[3 * i] * pp[3 * i + 1];
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const double nb = __shfl_down_sync(0xffffffffu, n, o), mb = __shfl_down_sync(0xffffffffu, m, o),
-                 m2b = __shfl_down_sync(0xffffffffu, m2, o);
-    chan_d(n, m, m2, nb, mb, m2b);
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+    s += __shfl_xor_sync(0xffffffffu, s, o);
   }
+  const double m = n > 0.0 ? s / n : 0.0;
+  for (int i = lane; i < nitems; i += 32) {
+    const double d = pp[3 * i + 1] - m;
+    m2 += pp[3 * i + 2] + pp[3 * i] * (d * d);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
   if (lane == 0) {
     const double sd = n > 0.0 ? sqrt(fmax(m2 / n, 0.0)) : 0.0;
     float* c = partial + (size_t)field * kMaxRowBlocks + kColorCoef;
