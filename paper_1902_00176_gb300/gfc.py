@@ -129,6 +129,8 @@ _SIGNATURES = {
 def lib() -> ctypes.CDLL:
     """Load ``libgfc.so`` (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lib_lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -190,7 +192,12 @@ def _tune_key(handle):
     return buf.value.decode()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # without a Stream object per call
+
+
 def _stream_ptr(device) -> int:
+    if _raw_stream is not None and device.index is not None:
+        return _raw_stream(device.index)
     return torch.cuda.current_stream(device).cuda_stream
 
 
@@ -219,6 +226,7 @@ class Plan:
         self.device = torch.device("cuda", torch.cuda.current_device() if device is None else
                                    torch.device(device).index or 0)
         self.H, self.W, self.C, self.batch, self.dtype = H, W, C, batch, dtype
+        self._shape = (batch, C, H, W)
         o = _Opts(H, W, C, batch, _DTYPES[dtype], pad, 1 if exact else 0, chunk, None, streams,
                   1 if column_fft else 0, 1 if block_items else 0)
         h = ctypes.c_void_p()
@@ -248,6 +256,8 @@ class Plan:
         _check(lib().gfc_plan_set_stream(self._h, ctypes.c_void_p(_stream_ptr(self.device))))
 
     def _check_field(self, t: torch.Tensor, name: str) -> torch.Tensor:
+        if t.dtype is self.dtype and t.shape == self._shape and t.device == self.device and t.is_contiguous():
+            return t
         t = _as_bchw(t)
         if not t.is_cuda or t.device != self.device:
             raise ValueError(f"{name} must be a CUDA tensor on {self.device}")
@@ -545,6 +555,9 @@ class RaggedPlan:
             _check(lib().gfc_plan_create_ragged(ctypes.byref(h), len(self.items), ctypes.cast(arr, ctypes.c_void_p),
                                                 _DTYPES[dtype]))
         self._h = h
+        ends = [o + C * H * W for (C, H, W), o in zip(self.items, self.offsets)]
+        gaps = [e for a, b in zip(ends, self.offsets[1:] + [self.total]) for e in range(a, b)]
+        self._gaps = torch.tensor(gaps, dtype=torch.int64, device=self.device) if gaps else None
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
@@ -556,6 +569,12 @@ class RaggedPlan:
             self.close()
         except Exception:
             pass
+
+    def _result(self):
+        """An array for a call's output: the calls write every item, so only the elements
+        between items are zeroed (zeroing it all was 79 us of 152 million elements)."""
+        out = torch.empty(self.total, dtype=self.dtype, device=self.device)
+        return out if self._gaps is None else out.index_fill_(0, self._gaps, 0)
 
     def empty(self):
         return torch.zeros(self.total, dtype=self.dtype, device=self.device)
@@ -588,22 +607,22 @@ class RaggedPlan:
 
     def solve_from_gradient(self, gx, gy, out=None):
         gx, gy = self._check_flat(gx, "gx"), self._check_flat(gy, "gy")
-        out = self.empty() if out is None else self._check_flat(out, "out")
+        out = self._result() if out is None else self._check_flat(out, "out")
         self._bind_stream()
         _check(lib().gfc_solve_from_gradient(self._h, gx.data_ptr(), gy.data_ptr(), out.data_ptr()))
         return out
 
     def solve_from_laplacian(self, lap, out=None):
         lap = self._check_flat(lap, "lap")
-        out = self.empty() if out is None else self._check_flat(out, "out")
+        out = self._result() if out is None else self._check_flat(out, "out")
         self._bind_stream()
         _check(lib().gfc_solve_from_laplacian(self._h, lap.data_ptr(), out.data_ptr()))
         return out
 
     def backward(self, grad_out, grad_gx=None, grad_gy=None):
         grad_out = self._check_flat(grad_out, "grad_out")
-        grad_gx = self.empty() if grad_gx is None else self._check_flat(grad_gx, "grad_gx")
-        grad_gy = self.empty() if grad_gy is None else self._check_flat(grad_gy, "grad_gy")
+        grad_gx = self._result() if grad_gx is None else self._check_flat(grad_gx, "grad_gx")
+        grad_gy = self._result() if grad_gy is None else self._check_flat(grad_gy, "grad_gy")
         self._bind_stream()
         _check(lib().gfc_backward(self._h, grad_out.data_ptr(), grad_gx.data_ptr(), grad_gy.data_ptr()))
         return grad_gx, grad_gy
