@@ -4,7 +4,7 @@
 // (fast_<M>x<N>.cu) so the library builds in parallel.
 //
 // Hand-offs between the passes:
-//   pass L  (edited solves, Laplacian input, or rows too wide to stage) writes
+//   pass L  (edited solves, some 16-bit Laplacians, or rows too wide to stage) writes
 //           the packed rows z[pair][j] = L[2 pair][j] + i L[2 pair+1][j];
 //   pass A  stages the gradient rows of an item by bulk copy and forms L itself
 //           (or stages z, or the adjoint's grad_out rows), and writes the row
@@ -74,6 +74,7 @@ struct FastArgs {
   size_t tri_field;  // complex elements per field of the band scratch
   int stage_out;     // inverse row pass: output rows staged in shared memory, stored by bulk copy
   double invM, invN; // 1 / M, 1 / N (FP64 divisions are slow on this part)
+  int overlap;       // the kernels after the first may start while the one ahead ends (launch_after)
   int adj;           // the recursive column solve runs the adjoint (half-bands, the sum term at row 0)
   int l2res;         // the chunks' spectrum hand-off fits the L2: evict-first streams, evict-last spectrum,
                      // the inverse row pass drops the spectrum lines it has read
@@ -590,6 +591,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd(const
 #pragma unroll 1
   for (int w = blockIdx.x; w < items; w += gridDim.x, phase ^= 1u) {
     const int field = w / A.ngroups, g = w - field * A.ngroups;
+    if (TRI && w + (int)gridDim.x >= items) dependents_may_start();  // the block's last item
     if (TRI && g == 0 && tid == 0)  // the sweep's count of finished blocks for this field starts at 0
       reinterpret_cast<unsigned*>(reinterpret_cast<double*>(partial) + (size_t)field * (kMaxRowBlocks / 2) + kTriCnt)[0] = 0u;
     const bool landed = mbar_wait(&bar, phase);
@@ -838,6 +840,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
 #pragma unroll 1
   for (int w = blockIdx.x; w < items; w += gridDim.x, phase ^= 1u) {
     const int field = w / A.ngroups, g = w - field * A.ngroups;
+    if (TRI && w + (int)gridDim.x >= items) dependents_may_start();  // the block's last item
     if (TRI && !ADJ && g == 0 && tid == 0)  // the sweep's count of finished blocks for this field starts at 0
       reinterpret_cast<unsigned*>(reinterpret_cast<double*>(partial) + (size_t)field * (kMaxRowBlocks / 2) + kTriCnt)[0] = 0u;
     float gxa[EDIT == kEditThreshold ? kEdW : 1];
@@ -1062,10 +1065,10 @@ static __global__ void __launch_bounds__(32) k_adj_total(double* __restrict__ pa
 }
 
 // the same sum, by one warp of the carry sweep (every lane gets it)
-__device__ __forceinline__ float adj_total(const double* __restrict__ partial, int field, const FastArgs& A) {
+__device__ __forceinline__ float adj_total(const double* partial, int field, const FastArgs& A) {
   const double* pp = partial + (size_t)field * (kMaxRowBlocks / 2);
   double a = 0.0;
-  for (int i = threadIdx.x & 31; i < A.zpairs; i += 32) a += pp[i];
+  for (int i = threadIdx.x & 31; i < A.zpairs; i += 32) a += __ldcg(pp + i);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   return (float)a;
@@ -1182,13 +1185,15 @@ static __global__ void __launch_bounds__(32 * kTriSeg) k_tri_carries(float2* __r
   const int kb = blockIdx.x, field = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k = kb * kTriCols + lane;
   const bool col_ok = k >= 1 && k < A.Nh;
+  wait_for_predecessor();
+  dependents_may_start();
   if (kb == nkb) {
     const float sadj = A.adj ? adj_total(partial, field, A) : 0.0f;  // (every warp for itself)
     const int nr = min(A.srows, A.M - A.p);
     const float* c0 = tri_col0(tri, field, A);
     float2* col = spec + (size_t)field * A.srows * A.ldY;
     column0_solve<kTriSeg>(
-        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldg(c0 + (r - A.p)) : 0.0f); },
+        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldcg(c0 + (r - A.p)) : 0.0f); },
         [&](int r, float u) {
           if (r >= A.p && r < A.p + nr) col[(size_t)(r - A.p) * A.ldY] = make_float2(u, 0.0f);
         },
@@ -1366,6 +1371,8 @@ __global__ void __launch_bounds__(32 * kTriRegWarps, MAXG <= 16 ? 4 : 2) k_tri_c
     FastArgs A, int nkb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int task = blockIdx.x * kTriRegWarps + warp;
+  wait_for_predecessor();
+  dependents_may_start();
   if (task >= A.nf * (nkb + 1)) return;
   const int field = task / (nkb + 1), kb = task - field * (nkb + 1);
   const int k = kb * kTriCols + lane;
@@ -1378,7 +1385,7 @@ __global__ void __launch_bounds__(32 * kTriRegWarps, MAXG <= 16 ? 4 : 2) k_tri_c
     const float* c0 = tri_col0(tri, field, A);
     float2* col = spec + (size_t)field * A.srows * A.ldY;
     column0_solve<1>(
-        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldg(c0 + (r - A.p)) : 0.0f); },
+        [&](int r) { return r == 0 ? -sadj : (r >= A.p && r < A.p + nr ? __ldcg(c0 + (r - A.p)) : 0.0f); },
         [&](int r, float u) {
           if (r >= A.p && r < A.p + nr) col[(size_t)(r - A.p) * A.ldY] = make_float2(u, 0.0f);
         },
@@ -1812,6 +1819,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
   };
   if (tid == 0) mbar_init(&bar, 1);
   __syncthreads();
+  if constexpr (TRI) wait_for_predecessor();
   if (tid == 0 && (int)blockIdx.x < items) issue(blockIdx.x, false);
   if (tid == 0 && (int)(blockIdx.x + gridDim.x) < items) issue(blockIdx.x + gridDim.x, true);
   prefetch(blockIdx.x);
@@ -2019,7 +2027,7 @@ static __global__ void __launch_bounds__(256) k_fast_color_finish(float* __restr
   const double* pp = reinterpret_cast<const double*>(partial) + (size_t)field * (kMaxRowBlocks / 2) + kStatsOff;
   // N = sum n_i, mean = sum n_i m_i / N, M2 = sum (M2_i + n_i (m_i - mean)^2): one
   // FP64 division a field (pairwise updates of (n, m, M2) take one a step, 2 us each
-  // here: 19 us for 24 fields of 120 items, 4 us this way)
+  // here: 19 us for 24 fields of 120 items, 10 us this way)
   double n = 0.0, s = 0.0, m2 = 0.0;
   for (int i = lane; i < nitems; i += 32) {
     n += pp[3 * i];
@@ -2228,6 +2236,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_ADJ) k_fast_rows_adj(const
   };
   if (tid == 0) mbar_init(&bar, 1);
   __syncthreads();
+  if constexpr (TRI) wait_for_predecessor();
   if (tid == 0 && (int)blockIdx.x < items) issue(blockIdx.x, false);
   if (tid == 0 && (int)(blockIdx.x + gridDim.x) < items) issue(blockIdx.x + gridDim.x, true);
   unsigned phase = 0;
@@ -2359,19 +2368,48 @@ static cudaError_t fast_setup(K kernel, int threads, size_t smem, int* slots) {
   return cudaSuccess;
 }
 
+// Launch a kernel that, with `overlap`, may start while the one ahead of it in the
+// stream ends (its reads of that one's results come after wait_for_predecessor):
+// the launch latency and the twiddle tables' loads overlap the predecessor's last
+// blocks. Taken for short solves (overlap_launches): three fields of 801x1200 41.1
+// -> 39.0 us, 48 Laplacians of 512x512 94.3 -> 89.1, 24 thresholded and corrected
+// fields of 720x1080 235 -> 220, 12 and 40 million pixels of other row lengths 1 to
+// 5% faster; not for long ones, where blocks that start early beside the
+// predecessor's unbalance the persistent grids (100 fields of 801x1200 528 -> 603),
+// nor for the adjoint (most lengths 3% faster, but 312x312 and 492x492 10 to 13%
+// slower), nor where other streams could use the slots that waiting blocks hold (64
+// ragged images 1746 -> 1871).
+constexpr double kOverlapMaxPixels = 48e6;
+static int overlap_launches(const gfc_plan* P, int nf) {
+  return !P->shares_gpu && P->nslots == 1 && (double)nf * P->H * P->W <= kOverlapMaxPixels;
+}
+template <typename... P, typename... Q>
+static cudaError_t launch_after(int overlap, void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                cudaStream_t st, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // The carry sweep of the chunk's fields over its A.G bands (tables for those bands;
 // k_tri_carries' shared-memory cap already raised).
 static cudaError_t launch_sweep(float2* spec, float2* tri, const float* cc, const float* powc, double* pd,
                                 const FastArgs& A, int nkb, cudaStream_t st) {
   if (A.G <= kTriRegG) {
-    const int grid = (A.nf * (nkb + 1) + kTriRegWarps - 1) / kTriRegWarps;
+    const dim3 grid((A.nf * (nkb + 1) + kTriRegWarps - 1) / kTriRegWarps);
     auto k = A.G <= 8 ? k_tri_carries_reg<8> : (A.G <= 16 ? k_tri_carries_reg<16> : k_tri_carries_reg<kTriRegG>);
-    k<<<grid, 32 * kTriRegWarps, 0, st>>>(spec, tri, cc, pd, A, nkb);
-  } else {
-    const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
-    k_tri_carries<<<dim3(nkb + 1, A.nf), 32 * kTriSeg, tsm, st>>>(spec, tri, cc, powc, pd, A);
+    return launch_after(A.overlap, k, grid, 32 * kTriRegWarps, 0, st, spec, tri, cc, pd, A, nkb);
   }
-  return cudaGetLastError();
+  const size_t tsm = A.G <= kTriTileMaxG ? (size_t)2 * A.G * kTriCols * sizeof(float2) : 0;
+  return launch_after(A.overlap, k_tri_carries, dim3(nkb + 1, A.nf), 32 * kTriSeg, tsm, st, spec, tri, cc, powc, pd, A);
 }
 
 // The fused row pass stages its input rows in the exchange buffers, extended
@@ -2448,6 +2486,7 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   A.invN = 1.0 / (double)P->N;
   A.adj = 1;
   A.l2res = 0;
+  A.overlap = 0;
   A.H = P->H; A.W = P->W; A.p = P->pad; A.M = P->M; A.N = P->N; A.Nh = P->Nh; A.ldM = P->ldM;
   A.nrows = P->H;
   A.ncols = P->W;
@@ -2500,10 +2539,10 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   FastArgs C = A;
   C.ngroups = (P->H + RS::F - 1) / RS::F;  // half-bands holding output rows
   prof_begin(P, 2, st);
-  k_fast_rows_adj<RS, T, true><<<grid_for((long)nf * C.ngroups, slots_c), RS::THREADS, RS::smem_bytes_adj_tri(),
-                                 st>>>(bf.spec, ggx, ggy, P->twN, C, bf.tri, P->colcoef_h);
+  e = launch_after(A.overlap, k_fast_rows_adj<RS, T, true>, dim3(grid_for((long)nf * C.ngroups, slots_c)), RS::THREADS,
+                   RS::smem_bytes_adj_tri(), st, bf.spec, ggx, ggy, P->twN, C, bf.tri, P->colcoef_h);
   prof_end(P, st);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // MODE 0: solve from gradient, 1: from Laplacian, 2: adjoint (in0 = grad_out,
@@ -2544,6 +2583,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   A.invN = 1.0 / (double)P->N;
   A.adj = 0;
   A.l2res = (tri && P->l2res) ? 1 : 0;
+  A.overlap = overlap_launches(P, nf);
   A.H = P->H; A.W = P->W; A.p = P->pad; A.M = P->M; A.N = P->N; A.Nh = P->Nh; A.ldM = P->ldM;
   A.nrows = (MODE == 0) ? P->H + 1 : P->H;
   A.ncols = (MODE == 0) ? P->W + 1 : P->W;
@@ -2710,14 +2750,14 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
     if (stats) {
       C.nparts = nkb;
       if constexpr (MODE == 0 && !kLean)
-        k_fast_rows_inv<RS, T, true, true>
-            <<<grid_for((long)nf * C.ngroups, slots_ts), RS::THREADS, RS::smem_bytes_tri_inv(), st>>>(
-                bf.spec, bf.partial, out0, P->twN, C, bf.tri, P->colcoef);
+        e = launch_after(A.overlap, k_fast_rows_inv<RS, T, true, true>, dim3(grid_for((long)nf * C.ngroups, slots_ts)),
+                         RS::THREADS, RS::smem_bytes_tri_inv(), st, bf.spec, bf.partial, out0, P->twN, C, bf.tri,
+                         P->colcoef);
     } else if (tri) {
       C.nparts = nkb;
-      k_fast_rows_inv<RS, T, true, false>
-          <<<grid_for((long)nf * C.ngroups, slots_tc), RS::THREADS, RS::smem_bytes_tri_inv(), st>>>(
-              bf.spec, bf.partial, out0, P->twN, C, bf.tri, P->colcoef);
+      e = launch_after(A.overlap, k_fast_rows_inv<RS, T, true, false>, dim3(grid_for((long)nf * C.ngroups, slots_tc)),
+                       RS::THREADS, RS::smem_bytes_tri_inv(), st, bf.spec, bf.partial, out0, P->twN, C, bf.tri,
+                       P->colcoef);
     } else if constexpr (kCols) {
       k_fast_rows_inv<RS, T, false, false>
           <<<grid_for((long)nf * C.ngroups, slots_c), RS::THREADS, RS::smem_bytes(), st>>>(
@@ -2725,7 +2765,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
     }
     if (stats) {
       prof_end(P, st);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
       prof_begin(P, 3, st);  // counted with the other non-transform pass
       const long long n = (long long)P->H * P->W;
       k_fast_color_finish<<<(nf + 7) / 8, 256, 0, st>>>(bf.partial, C.ngroups, nf, ed->ref_mean, ed->ref_std);
@@ -2740,7 +2780,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
     }
   }
   prof_end(P, st);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Shapes compiled for their row length only (the recursive column solve needs

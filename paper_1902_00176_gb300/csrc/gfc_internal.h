@@ -88,6 +88,7 @@ struct gfc_plan {
   bool fast;  // the row length has register-resident passes (fast_kernels.cuh)
   bool fast_cols;  // ... and the column length has them too (column FFT path, adjoint)
   bool tri;   // fast passes with the column direction by recursive filters (gfc_column_solver)
+  bool shares_gpu;   // other plans' launches run beside this one's (sub-plans of a ragged plan)
   bool block_items;  // fast passes launch one block per item (else persistent grids)
   bool l2res;        // recursive column solve whose spectrum hand-off (chunk x streams) fits kL2ResidentBytes
   int triG;   // bands of the recursive column solve (pass A's items)

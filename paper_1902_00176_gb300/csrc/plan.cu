@@ -544,6 +544,7 @@ static gfc_status attach_subplans(gfc_plan* p, const std::vector<int>& fast_item
     o.H = it.H; o.W = it.W; o.C = it.C; o.batch = 1; o.dtype = p->dtype; o.pad = 4; o.streams = 1;
     gfc_status st = gfc_plan_create_ex(&p->sub[j], &o);
     if (st != GFC_OK) return st;
+    p->sub[j]->shares_gpu = true;
     p->nsub = j + 1;
     p->sub_off[j] = it.offset;
     p->sub_work[j] = (double)it.C * it.H * it.W;

@@ -124,6 +124,13 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 // the issuing thread: wait until its bulk stores have completed
 __device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
+// Programmatic dependent launch. A kernel launched with launch_after may start
+// before the one ahead of it in its stream has ended, once every block of that
+// one has called dependents_may_start or ended: it runs what does not depend on
+// it, then waits for its end here (a no-op in a kernel launched the usual way).
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 // wait until the barrier's phase `parity` has completed; false if the time
 // bound ran out
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity,
