@@ -2502,8 +2502,10 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   A.G = P->triGh;       // the sweep's half-bands of F rows
   A.tri_field = P->tri_field;
   const int nkb = (P->Nh + kTriCols - 1) / kTriCols;
-  if ((size_t)2 * RS::F * A.ldY > (size_t)RS::F * RS::NP || A.zpairs > kAdjTotal ||
-      (size_t)A.srows * A.ldY > P->spec_field || nkb > kTriCnt)
+  // the row pairs' FP64 sums have kAdjTotal slots a field: taller images (above
+  // 2030 to 2045 rows) run the generic adjoint
+  if (A.zpairs > kAdjTotal) return cudaErrorNotSupported;
+  if ((size_t)2 * RS::F * A.ldY > (size_t)RS::F * RS::NP || (size_t)A.srows * A.ldY > P->spec_field || nkb > kTriCnt)
     return cudaErrorInvalidConfiguration;
   static std::mutex mu;
   static int slots_a = 0, slots_c = 0;
@@ -2600,7 +2602,8 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   A.G = P->triG;
   A.tri_field = P->tri_field;
   // the row passes stage their F packed rows / 2F rows of Y in the exchange buffer
-  if ((size_t)2 * RS::F * A.ldY > (size_t)RS::F * RS::NP || A.ldz > RS::NP || A.zpairs > kAdjTotal)
+  // (and the column-FFT adjoint sums grad_out per packed row, in kAdjTotal slots)
+  if ((size_t)2 * RS::F * A.ldY > (size_t)RS::F * RS::NP || A.ldz > RS::NP || (MODE == 2 && A.zpairs > kAdjTotal))
     return cudaErrorInvalidConfiguration;
   if (tri && (size_t)A.srows * A.ldY > P->spec_field) return cudaErrorInvalidConfiguration;
   if (tri && (P->Nh + kTriCols - 1) / kTriCols > kTriCnt) return cudaErrorInvalidConfiguration;
