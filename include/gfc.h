@@ -367,7 +367,8 @@ gfc_status gfc_solve_edited(gfc_plan* plan, const void* gx, const void* gy, cons
  * solved field, ref_mean / ref_std the original image's statistics (device
  * arrays of batch * C floats, e.g. from gfc_field_stats); a field with
  * std(I_c) = 0 becomes ref_mean. `edit` may be NULL (no edit) or as for
- * gfc_solve_edited. On plans with the recursive column solve the statistics of
+ * gfc_solve_edited. On plans with the recursive column solve (FP32 rows above the
+ * short lengths, images of up to 146 items of row pairs) the statistics of
  * I_c are taken while the last pass stores it (per-item FP64 partials, reduced
  * in a fixed order), and one more pass applies the correction in place: out is
  * written once by the solve and read and written once more. Other plans run the

@@ -1744,9 +1744,8 @@ __device__ __forceinline__ void tri_load_pair(float2 (&v)[S::R1], const float2* 
 }
 
 // Per-field statistics of the stored output (colour correction, Eq. 25): item
-// g of a field writes (sum x, sum x^2) of its stored values in FP64 at
-// partial (as doubles) + field * kMaxRowBlocks / 2 + kStatsOff + 2 g.
-constexpr int kStatsOff = 160;
+// g of a field writes (n, mean, sum of squared deviations) of its stored values in
+// FP64 at partial (as doubles) + field * kMaxRowBlocks / 2 + kStatsOff + 3 g.
 
 template <class S, typename T, bool TRI, bool STATS>
 __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const float2* __restrict__ Y,
@@ -2017,8 +2016,6 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_INV) k_fast_rows_inv(const
 // writes (mean, gain = ref_std / std or 0 when std = 0, ref_mean) at
 // kColorCoef of the field's scratch. k_fast_color_apply maps
 // x <- (x - mean) gain + ref_mean, 16 bytes per access where the field allows.
-constexpr int kColorCoef = 1200;  // float offset (past the item statistics, 3 doubles per item)
-
 static __global__ void __launch_bounds__(256) k_fast_color_finish(float* __restrict__ partial, int nitems, int nf,
                                                                   const float* __restrict__ ref_mean,
                                                                   const float* __restrict__ ref_std) {
@@ -2556,7 +2553,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
                                  cudaStream_t st, const EditArgs* ed = nullptr) {
   constexpr bool kCols = !std::is_same_v<CS, NoCols>;  // column transforms compiled for this shape
   // the short lengths and 16-bit storage on the lengths compiled for their rows
-  // only: edits go through pass L and there are no statistics (fast_rows_lean);
+  // only: edits go through pass L and there are no statistics (fast_rows_stats);
   // in 16 bits Laplacians go through pass L too and nothing is solved in one
   // launch (half the kernels of a length, of two types)
   constexpr bool kLean16 = !kCols && sizeof(T) == 2;
@@ -2748,8 +2745,7 @@ static cudaError_t run_fast_mode(gfc_plan* P, const Bufs& bf, const T* in0, cons
   } else {
     (void)out1;
     C.ngroups = ((P->H + 1) / 2 + RS::F - 1) / RS::F;
-    const bool stats = MODE == 0 && !kLean && tri && ed && ed->ref_mean;
-    if (stats && (kStatsOff + 3 * C.ngroups > kColorCoef / 2 || nkb > kStatsOff)) return cudaErrorInvalidConfiguration;
+    const bool stats = MODE == 0 && !kLean && tri && ed && ed->ref_mean;  // (fast_rows_stats)
     if (stats) {
       C.nparts = nkb;
       if constexpr (MODE == 0 && !kLean)

@@ -165,6 +165,10 @@ struct gfc_plan {
 namespace gfc {
 
 constexpr int kMaxRowBlocks = 2048;
+// the inverse row pass's statistics (corrected solves) in a field's partial-sum
+// area: three doubles per item from double kStatsOff, up to the colour
+// coefficients at float kColorCoef
+constexpr int kStatsOff = 160, kColorCoef = 1200;
 
 // thread-local error text, set by fail()
 gfc_status fail(gfc_status s, const char* fmt, ...);
@@ -189,9 +193,10 @@ cudaError_t build_colcoef(float* cc, float* pw, int M, int N, int Nh, int ldY, i
 // register-resident passes (solve_fast.cu): spectrum laid out [l][r]
 bool fast_supported(int M, int N);      // row and column passes compiled for M x N
 bool fast_rows_supported(int M, int N);  // row passes for N with the recursive column solve (of length M)
-// plans on the short and the long lengths, and 16-bit plans, compiled without column passes: no
-// statistics in the inverse row pass (gfc_solve_corrected runs them as separate passes)
-bool fast_rows_lean(int M, int N, gfc_dtype dtype);
+// whether a plan's inverse row pass can take the statistics of gfc_solve_corrected (else they are
+// separate passes): not on the short and the long lengths, nor in 16 bits where no column passes are
+// compiled, nor for more items a field than there is room for
+bool fast_rows_stats(const gfc_plan* P);
 int fast_row_lengths(int* out, int cap);  // compiled row lengths, ascending; returns the count
 size_t fast_zbuf_elems(int H, int M, int N);  // per field
 int fast_row_items(int M, int N);             // row pairs per item of the row passes (F)

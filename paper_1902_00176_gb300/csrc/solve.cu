@@ -873,7 +873,7 @@ gfc_status gfc_solve_corrected(gfc_plan* plan, const void* gx, const void* gy, c
   if (out == gx || out == gy || (edit && out == edit->edges))
     return fail(GFC_ERR_INVALID_ARG, "gfc_solve_corrected: out aliases an input");
   if (plan->ragged) return fail(GFC_ERR_UNSUPPORTED, "gfc_solve_corrected: ragged plans are not supported");
-  if (plan->fast && plan->tri && !plan->exact && !fast_rows_lean(plan->M, plan->N, plan->dtype)) {
+  if (fast_rows_stats(plan)) {
     EditArgs ed;
     if (gfc_status s = prepare_edit(plan, gx, gy, edit, &ed, "gfc_solve_corrected")) return s;
     ed.ref_mean = ref_mean;

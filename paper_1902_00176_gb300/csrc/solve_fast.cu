@@ -82,9 +82,13 @@ bool fast_rows_supported(int M, int N) {
   return find_rows(N) != nullptr || find_by_rows(N) != nullptr || long_rows_supported(M, N);
 }
 
-bool fast_rows_lean(int M, int N, gfc_dtype dtype) {
-  if (find(M, N) != nullptr) return false;
-  return ((dtype != GFC_F32 || N <= kRowPolicyMin) && find_rows(N) != nullptr) || long_rows_supported(M, N);
+bool fast_rows_stats(const gfc_plan* P) {
+  if (!P->fast || !P->tri || P->exact) return false;
+  const int F = fast_row_items(P->M, P->N), items = ((P->H + 1) / 2 + F - 1) / F;
+  if (kStatsOff + 3 * items > kColorCoef / 2) return false;  // 146 items: to 584 rows at F = 2, 2920 at F = 10
+  if (find(P->M, P->N) != nullptr) return true;
+  if (find_rows(P->N) != nullptr) return P->dtype == GFC_F32 && P->N > kRowPolicyMin;
+  return find_by_rows(P->N) != nullptr;
 }
 
 int fast_row_lengths(int* out, int cap) {  // the listed lengths that have a kernel set
