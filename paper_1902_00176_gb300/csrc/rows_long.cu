@@ -285,6 +285,32 @@ __global__ void __launch_bounds__(kLongThreads, 2) k_long_inv(const float2* S, c
   }
 }
 
+// Shared memory of a block, and the most that any length takes (N = 4096).
+size_t long_smem(const LongPlan& L) { return ((size_t)kLongF * L.len + tw_slot(L.n)) * sizeof(float2); }
+constexpr int kLongSmemMax = 104448;
+
+// Raise the kernels' shared-memory limits, once per device and storage type, to
+// what the longest rows need: the attribute is set, not raised, and the modes
+// share the inverse kernel, so a limit set by length would lower another plan's.
+template <typename T>
+cudaError_t long_setup(int device) {
+  constexpr int kDevices = 64;
+  static std::mutex mu;
+  static bool ready[kDevices] = {};
+  std::lock_guard<std::mutex> lock(mu);
+  const bool known = device >= 0 && device < kDevices;
+  if (known && ready[device]) return cudaSuccess;
+  auto raise = [](auto kernel, int bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  cudaError_t e = raise(k_long_fwd<T, 0>, kLongSmemMax);
+  if (e == cudaSuccess) e = raise(k_long_fwd<T, 1>, kLongSmemMax);
+  if (e == cudaSuccess) e = raise(k_long_inv<T>, kLongSmemMax);
+  if (e == cudaSuccess) e = raise(k_tri_carries, (int)((size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2)));
+  if (e == cudaSuccess && known) ready[device] = true;
+  return e;
+}
+
 template <typename T, int MODE>
 cudaError_t run_long(gfc_plan* P, const Bufs& bf, const T* in0, const T* in1, T* out, int nf, cudaStream_t st) {
   LongPlan L;
@@ -311,26 +337,11 @@ cudaError_t run_long(gfc_plan* P, const Bufs& bf, const T* in0, const T* in1, T*
   A.tri_field = P->tri_field;
   const int nkb = (P->Nh + kTriCols - 1) / kTriCols;
   if ((size_t)A.srows * A.ldY > P->spec_field || nkb > kTriCnt) return cudaErrorInvalidConfiguration;
-  const size_t smem = ((size_t)kLongF * L.len + tw_slot(L.n)) * sizeof(float2);
+  const size_t smem = long_smem(L);
+  if (smem > (size_t)kLongSmemMax) return cudaErrorInvalidConfiguration;
   double* pd = reinterpret_cast<double*>(bf.partial);
-  cudaError_t e;
-  {
-    static std::mutex mu;
-    static size_t cap = 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (smem > cap) {
-      if ((e = cudaFuncSetAttribute(k_long_fwd<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-          cudaSuccess)
-        return e;
-      if ((e = cudaFuncSetAttribute(k_long_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-          cudaSuccess)
-        return e;
-      if ((e = cudaFuncSetAttribute(k_tri_carries, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)((size_t)2 * kTriTileMaxG * kTriCols * sizeof(float2)))) != cudaSuccess)
-        return e;
-      cap = smem;
-    }
-  }
+  cudaError_t e = long_setup<T>(P->device);
+  if (e != cudaSuccess) return e;
   prof_begin(P, 0, st);
   k_long_fwd<T, MODE><<<(unsigned)((long)nf * A.G), kLongThreads, smem, st>>>(in0, in1, bf.spec, P->twN, pd, A, L,
                                                                               bf.tri, P->colcoef);

@@ -96,3 +96,26 @@ def test_edits_and_correction_on_long_rows():
     p.color_correct(two, m, s)
     assert torch.equal(one, two)
     p.close()
+
+
+def _call(p, mode, a, b):
+    return p.solve_from_gradient(a, b) if mode == "gradient" else p.solve_from_laplacian(a)
+
+
+@pytest.mark.parametrize("dt", [F32, BF16])
+def test_widths_and_modes_interleaved(dt):
+    """Plans kept side by side: a call of one width and input form does not change what
+    another may launch, whichever came first, and its bits stay the same."""
+    rng = np.random.default_rng(9650)
+    t = lambda W: torch.from_numpy(rng.standard_normal((1, 1, 30, W)).astype(np.float32)).to(DEV).to(dt)  # noqa: E731
+    wide, narrow = gfc.Plan(30, 4088, dtype=dt, device=DEV), gfc.Plan(30, 2092, dtype=dt, device=DEV)
+    ins = {p: (t(p.W), t(p.W)) for p in (wide, narrow)}
+    order = [(wide, "gradient"), (narrow, "laplacian"), (wide, "gradient"), (wide, "laplacian"), (narrow, "gradient"),
+             (wide, "laplacian"), (wide, "gradient")]
+    first = {}
+    for p, mode in order:
+        out = _call(p, mode, *ins[p])
+        torch.cuda.synchronize()
+        assert torch.equal(out, first.setdefault((p, mode), out))
+    wide.close()
+    narrow.close()
