@@ -543,7 +543,8 @@ static gfc_status run_all(gfc_plan* P, const void* a, const void* b, void* o0, v
     for (int s = 0; s < P->nslots; ++s) GFC_CUDA_TRY(cudaStreamWaitEvent(P->slot_stream[s], P->ev_fork, 0));
   }
   long c = 0;
-  for (long f0 = 0; f0 < fields; f0 += P->chunk, ++c) {
+  cudaError_t e = cudaSuccess;
+  for (long f0 = 0; f0 < fields && e == cudaSuccess; f0 += P->chunk, ++c) {
     const int nf = (int)((fields - f0 < P->chunk) ? fields - f0 : P->chunk);
     const T* in0 = static_cast<const T*>(a) + f0 * fe;
     const T* in1 = b ? static_cast<const T*>(b) + f0 * fe : nullptr;
@@ -560,17 +561,16 @@ static gfc_status run_all(gfc_plan* P, const void* a, const void* b, void* o0, v
         ec.ref_std += f0;
       }
     }
-    cudaError_t e = run_chunk<T, MODE>(P, slot_bufs(P, s), in0, in1, out0, out1, nf,
-                                       fork ? P->slot_stream[s] : P->stream, ed ? &ec : nullptr);
-    if (e != cudaSuccess) return cuda_fail(e, "gfc solve launch");
+    e = run_chunk<T, MODE>(P, slot_bufs(P, s), in0, in1, out0, out1, nf, fork ? P->slot_stream[s] : P->stream,
+                           ed ? &ec : nullptr);
   }
-  if (fork) {
+  if (fork) {  // (after a failed chunk too: the chunks queued before it use the caller's arrays)
     for (int s = 0; s < P->nslots; ++s) {
       GFC_CUDA_TRY(cudaEventRecord(P->slot_done[s], P->slot_stream[s]));
       GFC_CUDA_TRY(cudaStreamWaitEvent(P->stream, P->slot_done[s], 0));
     }
   }
-  return GFC_OK;
+  return e == cudaSuccess ? GFC_OK : cuda_fail(e, "gfc solve launch");
 }
 
 // Ragged batches: per chunk of fields, each pass is one launch over all its
@@ -664,19 +664,19 @@ static gfc_status run_ragged_subplans(gfc_plan* P, const void* a, const void* b,
   };
   GFC_CUDA_TRY(cudaEventRecord(P->rag_fork, P->stream));
   for (int s = 0; s < P->rag_active; ++s) GFC_CUDA_TRY(cudaStreamWaitEvent(P->rag_stream[s], P->rag_fork, 0));
-  for (int j = 0; j < P->nsub; ++j) {
+  gfc_status st = GFC_OK;
+  for (int j = 0; j < P->nsub && st == GFC_OK; ++j) {
     gfc_plan* Q = P->sub[j];
     Q->stream = P->rag_stream[P->sub_stream[j]];
     const long long off = P->sub_off[j];
-    gfc_status st = dispatch<MODE>(Q, at(a, off), at(b, off), const_cast<void*>(at(o0, off)),
-                                   const_cast<void*>(at(o1, off)));
-    if (st != GFC_OK) return st;
+    st = dispatch<MODE>(Q, at(a, off), at(b, off), const_cast<void*>(at(o0, off)), const_cast<void*>(at(o1, off)));
   }
+  // joined after a failed item too: the caller's arrays are in use by the items queued before it
   for (int s = 0; s < P->rag_active; ++s) {
     GFC_CUDA_TRY(cudaEventRecord(P->rag_done[s], P->rag_stream[s]));
     GFC_CUDA_TRY(cudaStreamWaitEvent(P->stream, P->rag_done[s], 0));
   }
-  return GFC_OK;
+  return st;
 }
 
 template <int MODE>
