@@ -147,8 +147,13 @@ gfc_status gfc_plan_create_ex(gfc_plan** plan, const gfc_plan_opts* opts);
  * solved exactly as by a uniform plan of its own size: Eq. 3, Eq. 23,
  * Algorithm B, pad 4, SMOOTH sizes). Items may share or differ in size; one
  * Green spectrum and one pair of twiddle tables is built per distinct padded
- * size. Fields are processed in chunks that keep the spectrum scratch within
- * 1 GB; every pass of a chunk is one launch over all its fields. The solve,
+ * size. Items with register-resident row passes run as plans of their own on
+ * internal streams. The fields of the others are processed in chunks that keep
+ * the spectrum scratch within 1 GB, every pass of a chunk one launch over all
+ * its fields; so are items of fewer than 300 000 pixels (C H W) in 16 bits
+ * and, in FP32, images of at most 262 x 120, where a batch has four or more
+ * of them: those equal a uniform plan's result to FP32 rounding, the others
+ * bit for bit. The solve,
  * Laplacian and backward entry points take the packed arrays (each item at
  * its offset). gfc_plan_padded_size reports the largest M and N.
  * gfc_solve_from_gradient_host is not supported on ragged plans. Synchronous. */

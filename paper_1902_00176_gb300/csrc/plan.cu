@@ -526,7 +526,21 @@ static gfc_status create_ragged_generic(gfc_plan** out, int n, const gfc_item* i
 
 // Ragged plans: items whose padded size has register-resident row passes
 // run as uniform sub-plans (batch 1, the item's C) on internal streams; the
-// others go through the generic per-field passes.
+// others go through the generic per-field passes, and so do small items in 16
+// bits and FP32 thumbnails (short rows, columns too), where there are several. A sub-plan
+// costs three launches, 8 us of host time an item, and 0.14 ms to create; the
+// generic passes about 28 ps a pixel and three launches for all items: they meet
+// near 300 000 pixels (C H W). 64 items in BF16, us by sub-plans / generic:
+// 1x64x64 413 / 59, 3x128x128 449 / 177, 3x240x240 505 / 393, 1x512x512 543 / 477,
+// 3x320x320 636 / 633, 3x400x400 548 / 773, 3x512x512 649 / 1293; FP32 3x64x64 323 /
+// 104, 3x96x96 348 / 155. Up to three small items are as fast by sub-plans.
+// Other FP32 items keep a sub-plan at any size: the generic adjoint is 5 times (geometric
+// mean) further from 64 bits on long rows and more on long columns; on thumbnails 3
+// times, of 1e-6.
+constexpr double kRagSubplanPixels = 3.0e5;
+constexpr int kRagSmallRows = 270;
+constexpr size_t kRagSmallTogether = 4;
+
 static gfc_status attach_subplans(gfc_plan* p, const std::vector<int>& fast_items, const gfc_item* items) {
   const int ns = (int)fast_items.size();
   p->nsub = 0;
@@ -560,7 +574,7 @@ gfc_status gfc_plan_create_ragged(gfc_plan** out, int n, const gfc_item* items, 
   *out = nullptr;
   if (dtype != GFC_F32 && dtype != GFC_F16 && dtype != GFC_BF16)
     return fail(GFC_ERR_INVALID_ARG, "gfc_plan_create_ragged: unknown dtype %d", (int)dtype);
-  std::vector<int> fast_items, generic_items;
+  std::vector<int> fast_items, generic_items, small_items;
   int maxM = 0, maxN = 0, maxH = 0, maxW = 0;
   long long nfields = 0, rag_total = 0;
   for (int i = 0; i < n; ++i) {
@@ -576,9 +590,13 @@ gfc_status gfc_plan_create_ragged(gfc_plan** out, int n, const gfc_item* items, 
     // (the sub-plans' entry points take 16-byte aligned fields)
     const bool fast = getenv("GFC_FORCE_GENERIC") == nullptr && fast_rows_supported(M, N) &&
                       it.offset * (long long)dtype_size(dtype) % 16 == 0;
-    if (fast) fast_items.push_back(i);
-    else generic_items.push_back(i);
+    const bool small = (double)it.C * it.H * it.W < kRagSubplanPixels &&
+                       (dtype != GFC_F32 || (N <= kRowPolicyMin && M <= kRagSmallRows && !fast_supported(M, N)));
+    (fast ? (small ? small_items : fast_items) : generic_items).push_back(i);
   }
+  std::vector<int>& to = small_items.size() < kRagSmallTogether ? fast_items : generic_items;
+  to.insert(to.end(), small_items.begin(), small_items.end());
+  std::sort(to.begin(), to.end());
   if (nfields > (1 << 24)) return fail(GFC_ERR_UNSUPPORTED, "gfc_plan_create_ragged: too many fields");
   gfc_plan* p = nullptr;
   if (!generic_items.empty()) {
