@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
 #pragma unroll 1
   for (int w = blockIdx.x; w < items; w += gridDim.x, phase ^= 1u) {
     const int field = w / A.ngroups, g = w - field * A.ngroups;
-    if (TRI && w + (int)gridDim.x >= items) dependents_may_start();  // the block's last item
+    if (TRI && !ADJ && w + (int)gridDim.x >= items) dependents_may_start();  // the block's last item
     if (TRI && !ADJ && g == 0 && tid == 0)  // the sweep's count of finished blocks for this field starts at 0
       reinterpret_cast<unsigned*>(reinterpret_cast<double*>(partial) + (size_t)field * (kMaxRowBlocks / 2) + kTriCnt)[0] = 0u;
     float gxa[EDIT == kEditThreshold ? kEdW : 1];
@@ -884,8 +884,8 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_FWD) k_fast_rows_fwd_div(c
       const float t2 = t2s[field];
       const int r0 = g * RW, nx = (A.H - r0) < RW ? (A.H - r0) : RW;
       const T zero = f_from_f<T>(0.0f);
-      // staged pixels (r0 + i, j): gx in sgx row i, gy in sgy row i + 1; rows are
-      // 16-byte multiples, so 16 bytes (VE pixels) at a time
+      // staged pixels (r0 + i, j): gx in sgx row i, gy in sgy row i + 1; 16 bytes (VE
+      // pixels) at a time where rows are 16-byte multiples
       constexpr int VE = 16 / (int)sizeof(T);
       const int wv = A.W / VE;
       if (A.W % VE != 0) {  // rows at odd remainders: one pixel at a time
@@ -2173,7 +2173,8 @@ __device__ __forceinline__ void tri_solve_half_rows(float2* stg, const float2* c
 // TRI: the recursive column solve's adjoint; Y is then the row-major spectrum
 // S of Crop^T(grad_out) (srows rows per field), an item is half-band g (output
 // rows gF .. gF + F - 1), whose F + 1 rows of S and two carries arrive by bulk
-// copy and are solved in place (tri_solve_half) before the output transforms.
+// copy and are solved before the output transforms, into their inputs
+// (tri_solve_half) or in place (tri_solve_half_rows): see PACK_ADJ.
 template <class S, typename T, bool TRI = false>
 __global__ void __launch_bounds__(S::THREADS, S::MINB_ADJ) k_fast_rows_adj(const float2* __restrict__ Y, T* __restrict__ ggx,
                                                                  T* __restrict__ ggy, const float2* __restrict__ twg,
@@ -2233,7 +2234,6 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB_ADJ) k_fast_rows_adj(const
   };
   if (tid == 0) mbar_init(&bar, 1);
   __syncthreads();
-  if constexpr (TRI) wait_for_predecessor();
   if (tid == 0 && (int)blockIdx.x < items) issue(blockIdx.x, false);
   if (tid == 0 && (int)(blockIdx.x + gridDim.x) < items) issue(blockIdx.x + gridDim.x, true);
   unsigned phase = 0;
@@ -2370,12 +2370,16 @@ static cudaError_t fast_setup(K kernel, int threads, size_t smem, int* slots) {
 // the launch latency and the twiddle tables' loads overlap the predecessor's last
 // blocks. Taken for short solves (overlap_launches): three fields of 801x1200 41.1
 // -> 39.0 us, 48 Laplacians of 512x512 94.3 -> 89.1, 24 thresholded and corrected
-// fields of 720x1080 235 -> 220, 12 and 40 million pixels of other row lengths 1 to
-// 5% faster; not for long ones, where blocks that start early beside the
-// predecessor's unbalance the persistent grids (100 fields of 801x1200 528 -> 603),
-// nor for the adjoint (most lengths 3% faster, but 312x312 and 492x492 10 to 13%
-// slower), nor where other streams could use the slots that waiting blocks hold (64
-// ragged images 1746 -> 1871).
+// fields of 720x1080 235 -> 220. With it / without, over ten row lengths from 64 to
+// 1960, solves and Laplacians in FP32 and BF16, geometric mean (least to most): 12
+// million pixels 0.956 (0.90 to 1.005), 24 0.982 (0.94 to 1.028), 36 0.987 (0.97 to
+// 1.034), 48 0.987 (0.97 to 1.006), 64 0.989 (0.975 to 1.006), 80 0.990, 100 0.993;
+// the ones above 1.01 are N = 1250 at 24 and 36 million. Not for long ones, where it
+// gives 1% at most lengths but blocks that start early beside the predecessor's can
+// unbalance the persistent grids (100 fields of 801x1200 529 -> 609 us), nor for the
+// adjoint (most lengths 3% faster, but 312x312 and 492x492 10 to 13% slower), nor where
+// other streams could use the slots that waiting blocks hold (64 ragged images 1746 ->
+// 1871).
 constexpr double kOverlapMaxPixels = 48e6;
 static int overlap_launches(const gfc_plan* P, int nf) {
   return !P->shares_gpu && P->nslots == 1 && (double)nf * P->H * P->W <= kOverlapMaxPixels;
@@ -2467,11 +2471,12 @@ namespace gfc {
 // transpose of the solve, z = Crop^T(grad_out) - (sum grad_out) e_00 through
 // the same Green operator, then the forward differences' transposes): the
 // forward row pass packs grad_out into z's rows (row-pair sums for the e_00
-// term) and stores S with half-band sums; one warp per field reduces the sum;
-// the carry sweep runs over the half-bands with -sum at torus row 0; the
-// adjoint's inverse row pass solves each half-band in shared memory and writes
-// grad_gx, grad_gy. Needs grad_out rows that fit the forward pass's staging;
-// returns cudaErrorNotSupported otherwise.
+// term) and stores S with half-band sums; the carry sweep runs over the
+// half-bands with -sum at torus row 0, each of its blocks (warps) reducing the
+// row pairs' sums for itself; the adjoint's inverse row pass solves each
+// half-band in shared memory and writes grad_gx, grad_gy. Needs grad_out rows
+// that fit the forward pass's staging and at most kAdjTotal row pairs; returns
+// cudaErrorNotSupported otherwise.
 template <class RS, typename T>
 static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, T* ggx, T* ggy, int nf,
                                     cudaStream_t st) {
@@ -2538,10 +2543,10 @@ static cudaError_t run_fast_adj_tri(gfc_plan* P, const Bufs& bf, const T* gout, 
   FastArgs C = A;
   C.ngroups = (P->H + RS::F - 1) / RS::F;  // half-bands holding output rows
   prof_begin(P, 2, st);
-  e = launch_after(A.overlap, k_fast_rows_adj<RS, T, true>, dim3(grid_for((long)nf * C.ngroups, slots_c)), RS::THREADS,
-                   RS::smem_bytes_adj_tri(), st, bf.spec, ggx, ggy, P->twN, C, bf.tri, P->colcoef_h);
+  k_fast_rows_adj<RS, T, true><<<grid_for((long)nf * C.ngroups, slots_c), RS::THREADS, RS::smem_bytes_adj_tri(),
+                                 st>>>(bf.spec, ggx, ggy, P->twN, C, bf.tri, P->colcoef_h);
   prof_end(P, st);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return cudaGetLastError();
 }
 
 // MODE 0: solve from gradient, 1: from Laplacian, 2: adjoint (in0 = grad_out,

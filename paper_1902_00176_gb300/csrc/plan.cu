@@ -330,11 +330,11 @@ gfc_status gfc_plan_create_ex(gfc_plan** out, const gfc_plan_opts* o) {
   int nslots = o->streams;
   if (nslots == 0) nslots = 1;
   if (chunk == 0) {
-    // Measured on GB300 (801x1200 fields): the passes are bound by arithmetic
-    // and latency rather than by where the intermediates live, and large
-    // grids beat L2-sized chunks (1.11 ms per 100 fields in one chunk, 1.29 -
-    // 1.41 ms with 2 - 12 field chunks on 2 - 4 streams). So one chunk holds as
-    // many fields as 2 GB of scratch allows.
+    // One chunk of as many fields as 2 GB of scratch allows: the passes are
+    // bound by arithmetic and latency rather than by where the intermediates
+    // live. A split can be faster, by up to 5% (100 fields of 801x1200: 531 us
+    // in one chunk, 505 in chunks of 25 on four streams, whose sweeps and tails
+    // overlap the others' row passes); gfc_plan_autotune finds it.
     chunk = (long)((size_t(2) << 30) / (ws * nslots));
     if (chunk < 1) chunk = 1;
   }
@@ -362,8 +362,7 @@ gfc_status gfc_plan_create_ex(gfc_plan** out, const gfc_plan_opts* o) {
   if (e == cudaSuccess && p->tri)
     e = cudaMalloc(&p->colcoef_h, ((size_t)p->Nh * 8 + 2 * (size_t)p->ldS) * sizeof(float));
   if (e == cudaSuccess && p->tri) e = cudaMalloc(&p->powc_h, (size_t)tri_power_rows(p->triGh) * p->ldS * sizeof(float));
-  // (+64 bytes: the sweep's bulk copy of a field's column 0 rounds up to 16 bytes)
-  if (e == cudaSuccess && p->tri) e = cudaMalloc(&p->tri_buf, p->tri_field * chunk * nslots * sizeof(float2) + 64);
+  if (e == cudaSuccess && p->tri) e = cudaMalloc(&p->tri_buf, p->tri_field * chunk * nslots * sizeof(float2));
   for (int sl = 0; sl < nslots && e == cudaSuccess; ++sl) {
     e = cudaStreamCreateWithFlags(&p->slot_stream[sl], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->slot_done[sl], cudaEventDisableTiming);

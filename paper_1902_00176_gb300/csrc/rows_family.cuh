@@ -13,14 +13,15 @@ namespace gfc {
 // Row lengths: X(N, R1, R2, F), N = R1 R2 with R2 threads per transform and F
 // transforms per block (about 128 threads, within the shared memory of 2 forward
 // blocks and 3 inverse blocks per SM, 4 and 4 for N <= 512). Short lengths take
-// blocks of about 64 threads with few idle lanes, bands of at most 22 rows (their
-// column in registers) that a square image fills with little left over; each F is
+// blocks of about 64 threads with few idle lanes, bands of at most 22 rows (with
+// their recursions in registers up to 18, tri_solve_band) that a square image fills
+// with little left over; each F is
 // the faster of two to four tried, in ps a pixel of a solve: N = 42 F 16 23.8,
 // 9 14.6; 56 F 16 14.4, 8 11.6; 72 F 14 11.9, 7 9.2; 90 F 12 9.4, 6 8.2; 112 F 9
 // 7.2, 4 7.9. R2 dividing R1 keeps every thread in both stages and won wherever N
 // allows it at these sizes: 98 as 14 x 7 against 7 x 14 8.4 -> 6.6, 128 as 16 x 8
 // 7.4 -> 5.8, 882 as 42 x 21 6.8 -> 5.8 (adjoint 10.0 -> 8.2), 1200 as 60 x 20 6.8 ->
-// 6.35. Images narrower than 24 pixels (N < 32) keep the generic passes.
+// 6.35. Images narrower than 23 pixels (N < 32) keep the generic passes.
 #define GFC_ROWS_S(X)                                                                                        \
   X(32, 4, 8, 8) X(36, 6, 6, 5) X(40, 5, 8, 6) X(42, 6, 7, 9) X(48, 6, 8, 7) X(50, 5, 10, 11)            \
   X(54, 6, 9, 6) X(56, 7, 8, 8) X(60, 6, 10, 9) X(64, 8, 8, 8)
