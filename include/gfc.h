@@ -86,9 +86,9 @@ typedef enum { GFC_SIZE_SMOOTH = 0, GFC_SIZE_EXACT = 1 } gfc_size_policy;
  * two length-M transforms, no spectrum transpose. Used by solves, edited
  * solves and gfc_backward (which sweeps half-bands of rows so its inverse row
  * pass can produce one band of output rows per item; the -(sum grad_out) e_00
- * term enters the sweep and column 0 at torus row 0). Where the adjoint's
- * grad_out rows cannot be bulk-copied (W x element size not a multiple of 16
- * bytes) it runs the column transforms instead.
+ * term enters the sweep and column 0 at torus row 0). The adjoint runs
+ * column transforms instead on row lengths above 2058 and on images of more
+ * than 2030 to 2045 rows (by the row length).
  * GFC_COLUMN_FFT: column FFT, multiply by G, inverse column FFT. */
 typedef enum { GFC_COLUMN_RECURSIVE = 0, GFC_COLUMN_FFT = 1 } gfc_column_solver;
 
@@ -121,7 +121,9 @@ typedef struct {
  * GFC_ERR_UNSUPPORTED when M or N would exceed the largest supported length. */
 gfc_status gfc_padded_size(int H, int W, int pad, int size_policy, int* M, int* N);
 
-/* The row lengths N with register-resident row passes, ascending. Writes up to
+/* The row lengths N the SMOOTH policy draws from in its range, ascending; all
+ * have register-resident row passes (as have most even 7-smooth lengths from 32
+ * to 128 and from 2060 to 4096, the latter for solves). Writes up to
  * `capacity` of them to `lengths` (may be NULL when capacity is 0) and returns
  * how many there are. Host-only. */
 int gfc_row_lengths(int* lengths, int capacity);

@@ -158,7 +158,7 @@ def padded_size(H: int, W: int, pad: int = 4, exact: bool = False):
 
 
 def row_lengths():
-    """Row lengths N with register-resident row passes, ascending (host-only)."""
+    """Row lengths N the size policy draws from in its range, ascending (host-only)."""
     n = lib().gfc_row_lengths(None, 0)
     buf = (ctypes.c_int * n)()
     lib().gfc_row_lengths(buf, n)
